@@ -49,6 +49,26 @@ struct DState {                       // Eq. 1
   double qg[4];
 };
 
+// A frame's constants of the covariance-form step (joint_step.cuh), written when
+// the frame begins: offsets into Elim::m, and the frame's IMU pieces.
+constexpr int kElimPieces = 64;       // IMU pieces that step keeps in shared memory
+constexpr int kElPy = 0;              // 11 x 11: covariance P of x0's non-pose part y given its pose
+constexpr int kElK = 121;             // 11 x 6: y's mean by the pose
+constexpr int kElM0 = 187;            // 11: P b_y
+constexpr int kElHp = 198;            // 6 x 6: prior on the pose, y marginalised
+constexpr int kElBp = 234;            // 6: its vector
+constexpr int kElS6 = 240;            // 6 x 6: covariance of e_IMU's position and rotation rows
+constexpr int kElSv = 276;            // 3 x 6: its velocity rows against those
+constexpr int kElSg = 294;            // gravity row variance
+constexpr int kElT = 295;             // interval, s
+constexpr int kElimDoubles = 296;
+struct Elim {
+  int32_t ok;                         // 1: usable for this frame
+  int32_t np;                         // pieces
+  double m[kElimDoubles];
+  double piece[kElimPieces][8];       // dt, dt / 2, gyro (3), accelerometer (3)
+};
+
 struct Ctrl {
   // ---- result head: copied to the host after every frame ----
   DState x;                           // state after the last tracked frame
@@ -79,6 +99,7 @@ struct Ctrl {
   // (dR 9, dv 3, dp 3, Phi_g 9, V_g 9, P_g 9, V_a 9, P_a 9, T) and those biases
   double pre_lin[61];
   double b_lin[6];
+  Elim elim;
 };
 
 // Bytes of the result head (x .. pad1) copied back after each frame.

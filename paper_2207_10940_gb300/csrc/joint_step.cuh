@@ -1,0 +1,952 @@
+// The Gauss-Newton step of the joint problem with the non-pose unknowns
+// eliminated in covariance form (Eq. 6-7), for every iteration of a frame but
+// its last (which assembles the full system that marginalisation takes).
+//
+// What bounds a step is the FP64 pipe: on GB300 a warp's FP64 instruction holds
+// its sub-partition's pipe for 64 cycles whatever the number of active lanes
+// (measured: dependent DFMA 65 cycles, two independent ones 129; an f64 mma
+// m8n8k4 577, no faster per product; a 128-thread barrier 33, a shared-memory
+// exchange 35).  So the step is laid out to put the fewest FP64 instructions on
+// any one sub-partition along its chain, and this formulation needs far fewer
+// of them than the 26-variable information form:
+//
+//   unknowns     x0's pose p0 and x1's pose p1 (12), y = x0's velocity, biases
+//                and gravity (11), x1's velocity, biases and gravity (8).
+//   x1's velocity enters the velocity rows of e_IMU only (Jacobian -I) and no
+//                prior: it is free to follow, so those rows drop out and the
+//                position and rotation rows keep their own covariance block S6
+//                of Sigma (the marginal), fixed for the frame.
+//   x1's biases  follow x0's; x1's gravity leaves one row: along the normal n
+//                of its Jacobian block B, a dg0 + s with variance sigma_g^2.
+//   y            under the prior (H*, b*) given p0 is Gaussian with covariance
+//                P = H_yy^-1 and mean K p0 + m: P, K = -P H_yp, P b_y, and the
+//                Schur complement on p0 are fixed for the frame (k_frame_begin).
+//   so the 7 rows r = Jp p + Jy y + e become r' = (Jp + Jy K) p + (e + Jy m)
+//   with covariance S = blockdiag(S6, sigma_g^2) + Jy P Jy^T, and the system is
+//       [ -S   J' ] [ lambda ]   [ -e' ]
+//       [ J'^T H  ] [   p    ] = [  b  ]
+//   H, b: the prior on p0 plus the pixel terms.  The 7 multipliers are
+//   eliminated before the pixel sums arrive, the 12 poses after; then
+//   y = K p0 + m - P Jy^T lambda,  dv1 = e_v + J_v dx0 - S_v6 lambda.
+// This is the same minimiser as Eq. 7's in exact arithmetic; the 1e8-scale IMU
+// weights are never formed (their inverses are added instead).
+//
+// Measured against the information form (`gn_step_body`): a step on one block 102k ->
+// 66k cycles, one 640x480 camera 1207 -> 914 us per frame, 12 x 320x240 1471 -> 1110
+// us, 64 x 640x480 (steps hidden behind other groups' pixels) 4710 -> 4621 us.
+//
+// Included by solve.cu, inside its namespace, after the element-wise 3x3 algebra
+// and the warp-cooperative state algebra that it uses.
+
+template <int ID, int N>
+__device__ __forceinline__ void bar_sync() { asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(N) : "memory"); }
+template <int ID, int N>
+__device__ __forceinline__ void bar_arrive() { asm volatile("bar.arrive %0, %1;" ::"n"(ID), "n"(N) : "memory"); }
+
+// Pre-integration of a run of IMU pieces (and its derivatives by the biases):
+// rotation R, Phi = d(R)/d(b_g) (right perturbation), V = d(v)/d(b_g),
+// P = d(p)/d(b_g), Va, Pa by b_a, velocity v, position p, duration T.
+constexpr int kNR = 0, kNPhi = 9, kNV = 18, kNP = 27, kNVa = 36, kNPa = 45, kNv = 54, kNp = 57, kNT = 60;
+constexpr int kNode = 61;             // odd stride: consecutive nodes fall into different banks
+
+constexpr int kLam = 7, kPose = 12, kSys = kLam + kPose;      // 19 unknowns of the sweep
+constexpr int kSysEnt = kSys * (kSys + 1) / 2 + kSys;         // lower triangle + right-hand side row
+
+struct FastSmem {
+  double nodeA[kElimPieces][kNode];   // leaves, then every second level of the tree
+  double nodeB[kElimPieces / 2][kNode];
+  double X[kElimPieces / 2][18];      // V_2 - [v_2]x Phi_1 and P_2 - [p_2]x Phi_1 of each pair
+  double th[kElimPieces][3], t2[kElimPieces], ser[3][kElimPieces];
+  double piece[kElimPieces][8];       // as Elim::piece
+  double el[kElimDoubles];            // Elim's matrices
+  DState x0, x1, xbar;
+  double Rref[9];
+  double dx[34];                      // the step
+  // states only
+  double R0[9], Q0[9], R1[9], A0[9], QR[9], QA[9], RcR1T[9], c[3], t1[3], t2c[3], rcS[3], base[3], dr[3];
+  double d[17], m[11], bp[6];         // x0 boxminus xbar; mean of y; prior vector on p0
+  double eg[3], Jlg[9], Jrg[9], nv[3], mm[3], a[2], s, Gm[6], Ag[6];
+  double eb[6];                       // bias errors
+  double C[18][6];                    // pixel Jacobian maps: photometric on (p0, p1), ICP on p1
+  // after the pre-integration
+  double Jyr[3][11];                  // position rows by y
+  double RW[9], APg[9], t3[3], M[9], RP[9], t4[3], u[3], er[3], ea[3], Jla[9], Jra[9], B13[9];
+  double B14[9], B17[9], w9[3], t5[3], B9[9], B20[6], ev[3];
+  double T[kLam][11];                 // Jy P
+  double Jp[kLam][kPose];             // J'
+  double ep[kLam];                    // e'
+  double S[28];                       // S's lower triangle (without blockdiag(S6, sigma_g^2))
+  // pixel terms
+  double sums[kSumsAll];
+  double U[18][7];
+  double P12[kPose * kPose], g12[kPose];
+  // sweep
+  double col[2][kSys + 1];
+  double rinv[kSys], piv[kSys], z[kSys];
+  double L[kSys][kSys + 2];
+  double rot[18];
+  double fo[21];
+  double cost;
+  int good[2];
+};
+
+__device__ __forceinline__ int tri(int i, int j) { return i * (i + 1) / 2 + j; }   // i >= j
+
+// ---- IMU pieces --------------------------------------------------------------
+
+// Leaves of the pieces at biases (bg, ba): R = Exp(th), Phi = -Jr(th) dt, v = a dt,
+// p = a dt^2 / 2, Va = -dt I, Pa = -dt^2 / 2 I.  Warps 0-3.  The three series (or
+// sines) of a piece run on three lanes, its nine matrix elements on nine.
+__device__ void fast_leaves(FastSmem& S, int np, const double* bg, const double* ba) {
+  const int t = threadIdx.x;
+  for (int L = t; L < 6 * np; L += 128) {
+    const int q = L / np, k = L - q * np;
+    const double* pc = S.piece[k];
+    if (q < 3) {
+      S.th[k][q] = (pc[2 + q] - bg[q]) * pc[0];
+    } else {
+      const double v = (pc[2 + q] - ba[q - 3]) * pc[0];
+      S.nodeA[k][kNv + q - 3] = v;
+      S.nodeA[k][kNp + q - 3] = v * pc[1];
+    }
+  }
+  bar_sync<1, 128>();
+  for (int L = t; L < 3 * np; L += 128) {
+    const int q = L / np, k = L - q * np;
+    const double* w = S.th[k];
+    const double t2 = fma(w[0], w[0], fma(w[1], w[1], w[2] * w[2]));
+    double f;
+    if (t2 < kSeriesT2) {            // sin t / t, (1 - cos t) / t^2, (t - sin t) / t^3
+      const double c0 = q == 0 ? 1.0 : q == 1 ? 0.5 : 1.0 / 6;
+      const double c1 = q == 0 ? -1.0 / 6 : q == 1 ? -1.0 / 24 : -1.0 / 120;
+      const double c2 = q == 0 ? 1.0 / 120 : q == 1 ? 1.0 / 720 : 1.0 / 5040;
+      const double c3 = q == 0 ? -1.0 / 5040 : q == 1 ? -1.0 / 40320 : -1.0 / 362880;
+      const double c4 = q == 0 ? 1.0 / 362880 : q == 1 ? 1.0 / 3628800 : 1.0 / 39916800;
+      f = fma(t2, fma(t2, fma(t2, fma(t2, c4, c3), c2), c1), c0);
+    } else {
+      const double th = sqrt(t2);
+      double sn, cs;
+      sincos(th, &sn, &cs);
+      f = q == 0 ? sn / th : q == 1 ? (1.0 - cs) / t2 : (th - sn) / (t2 * th);
+    }
+    S.ser[q][k] = f;
+    if (q == 0) S.t2[k] = t2;
+  }
+  bar_sync<1, 128>();
+  for (int L = t; L < 9 * np; L += 128) {
+    const int k = L / 9, e = L - 9 * k, r = e / 3, c = e - 3 * r;
+    const double* w = S.th[k];
+    const double dt = S.piece[k][0], hdt = S.piece[k][1];
+    const double id = r == c ? 1.0 : 0.0;
+    const double K = hat_e(w, e), K2 = fma(w[r], w[c], r == c ? -S.t2[k] : 0.0);
+    const double ea = S.ser[0][k], eb = S.ser[1][k], jb = S.ser[2][k];
+    double* n = S.nodeA[k];
+    n[kNR + e] = fma(eb, K2, fma(ea, K, id));
+    n[kNPhi + e] = -dt * fma(jb, K2, fma(-eb, K, id));
+    n[kNV + e] = 0.0;
+    n[kNP + e] = 0.0;
+    n[kNVa + e] = r == c ? -dt : 0.0;
+    n[kNPa + e] = r == c ? -hdt * dt : 0.0;
+    if (e == 0) n[kNT] = dt;
+  }
+  bar_sync<1, 128>();
+}
+
+// Composition of two runs (1 then 2):
+//   R = R1 R2, Phi = R2^T Phi1 + Phi2, v = v1 + R1 v2, p = p1 + v1 T2 + R1 p2,
+//   V = V1 + R1 (V2 - [v2]x Phi1), P = P1 + V1 T2 + R1 (P2 - [p2]x Phi1),
+//   Va = Va1 + R1 Va2, Pa = Pa1 + Va1 T2 + R1 Pa2, T = T1 + T2
+// over a binary tree of the np leaves: ceil(log2 np) levels of 6 dependent FP64
+// instructions each, one output element per lane (the prefix scans and sums of
+// the sequential order take 14 dependent ones per sum besides the scans).
+// Warps 0-3; returns the root.
+__device__ const double* fast_tree(FastSmem& S, int np) {
+  const int t = threadIdx.x;
+  double(*in)[kNode] = S.nodeA;
+  double(*out)[kNode] = S.nodeB;
+  for (int n = np; n > 1; n = (n + 1) >> 1) {
+    const int full = n >> 1;
+    for (int L = t; L < 18 * full; L += 128) {
+      const int i = L / 18, e = L - 18 * i;
+      const double* n1 = in[2 * i];
+      const double* n2 = in[2 * i + 1];
+      const bool pos = e >= 9;
+      const int q = pos ? e - 9 : e, r = q / 3, c = q - 3 * r;
+      const int r1 = r == 2 ? 0 : r + 1, r2 = r == 0 ? 2 : r - 1;
+      const double* v = n2 + (pos ? kNp : kNv);
+      // minus row r of [v]x Phi1: -(v_r1 Phi_r2 - v_r2 Phi_r1)
+      S.X[i][e] = fma(v[r2], n1[kNPhi + 3 * r1 + c],
+                      fma(-v[r1], n1[kNPhi + 3 * r2 + c], n2[(pos ? kNP : kNV) + q]));
+    }
+    bar_sync<1, 128>();
+    for (int L = t; L < kNode * full; L += 128) {
+      const int i = L / kNode, e = L - kNode * i;
+      const double* n1 = in[2 * i];
+      const double* n2 = in[2 * i + 1];
+      double v;
+      if (e == kNT) {
+        v = n1[kNT] + n2[kNT];
+      } else {
+        const bool vec = e >= kNv;
+        const int f = vec ? (e - kNv) / 3 : e / 9;              // field
+        const int q = vec ? (e - kNv) - 3 * f : e - 9 * f;
+        const int r = vec ? q : q / 3, c = vec ? 0 : q - 3 * r;
+        const bool phi = !vec && f == 1;
+        const double* A = phi ? n2 + r : n1 + 3 * r;            // row r of R1, or of R2^T
+        const int sa = phi ? 3 : 1;
+        const double* B;
+        if (vec) B = n2 + (f == 0 ? kNv : kNp);
+        else if (f == 0) B = n2 + kNR + c;
+        else if (f == 1) B = n1 + kNPhi + c;
+        else if (f == 2 || f == 3) B = S.X[i] + (f == 2 ? 0 : 9) + c;
+        else B = n2 + (f == 4 ? kNVa : kNPa) + c;
+        const int sb = vec ? 1 : 3;
+        const double base = (!vec && f == 0) ? 0.0 : phi ? n2[e] : n1[e];
+        const bool lin = vec ? f == 1 : (f == 3 || f == 5);     // the T2-weighted velocity term
+        const double ve = lin ? n1[vec ? kNv + q : (f == 3 ? kNV : kNVa) + q] : 0.0;
+        v = fma(ve, n2[kNT], fma(A[0], B[0], fma(A[sa], B[sb], fma(A[2 * sa], B[2 * sb], base))));
+      }
+      out[i][e] = v;
+    }
+    if (n & 1)                       // the odd run out moves up unchanged
+      for (int e = t; e < kNode; e += 128) out[full][e] = in[n - 1][e];
+    bar_sync<1, 128>();
+    double(*s)[kNode] = in;
+    in = out;
+    out = s;
+  }
+  return in[0];
+}
+
+// First-order bias update (preint_first_order) into the node layout; warps 0-3.
+// Re-integrates (and moves the linearisation point) past the thresholds.
+__device__ const double* fast_first_order(const SolveParams& sp, Ctrl* c, FastSmem& S, int np) {
+  const int t = threadIdx.x;
+  const double* bg = S.x0.bg;
+  const double* ba = S.x0.ba;
+  double dbg[3], dba[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    dbg[i] = bg[i] - c->b_lin[i];
+    dba[i] = ba[i] - c->b_lin[3 + i];
+  }
+  const double ng = sqrt(dbg[0] * dbg[0] + dbg[1] * dbg[1] + dbg[2] * dbg[2]);
+  const double na = sqrt(dba[0] * dba[0] + dba[1] * dba[1] + dba[2] * dba[2]);
+  if (ng == 0.0 && na == 0.0) {                  // at the linearisation point: the integration itself,
+    fast_leaves(S, np, bg, ba);                  // the same bits as re-integrating every iteration
+    return fast_tree(S, np);
+  }
+  // pre_lin: dR 9, dv 3, dp 3, Phi_g 9, V_g 9, P_g 9, V_a 9, P_a 9, T
+  if (ng > sp.relin_g || na > sp.relin_a) {      // uniform over the warps
+    bar_sync<1, 128>();                          // every thread has read b_lin
+    fast_leaves(S, np, bg, ba);
+    const double* n = fast_tree(S, np);
+    if (t < 60) {
+      const int src = t < 9 ? kNR + t : t < 15 ? kNv + t - 9 : kNPhi + t - 15;   // Phi, V, P, Va, Pa follow
+      c->pre_lin[t] = n[src];
+    } else if (t == 60) {
+      c->pre_lin[60] = n[kNT];
+    } else if (t >= 64 && t < 70) {
+      c->b_lin[t - 64] = t < 67 ? bg[t - 64] : ba[t - 67];
+    }
+    return n;
+  }
+  const double* L = c->pre_lin;
+  double* n = S.nodeA[0];
+  double* th = S.fo;
+  double* E = S.fo + 3;
+  double* Jrm = S.fo + 12;
+  if (t < 3) {
+    th[t] = L[15 + 3 * t] * dbg[0] + L[16 + 3 * t] * dbg[1] + L[17 + 3 * t] * dbg[2];
+  } else if (t < 9) {
+    const int q = t - 3, i = q % 3;
+    const double* M = q < 3 ? L + 24 : L + 33;   // V_g or P_g
+    const double* N = q < 3 ? L + 42 : L + 51;   // V_a or P_a
+    double v = L[(q < 3 ? 9 : 12) + i];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) v = fma(M[3 * i + j], dbg[j], fma(N[3 * i + j], dba[j], v));
+    n[(q < 3 ? kNv : kNp) + i] = v;
+  } else if (t < 45) {
+    n[kNV + t - 9] = L[24 + t - 9];              // V_g, P_g, V_a, P_a
+  } else if (t == 45) {
+    n[kNT] = L[60];
+  }
+  bar_sync<1, 128>();
+  if (t < 9) {                                   // Exp(theta), Jr(theta): one element per lane
+    const double t2 = th[0] * th[0] + th[1] * th[1] + th[2] * th[2];
+    double ea, eb, jb;
+    if (t2 < kSeriesT2) {
+      ea = 1.0 + t2 * (-1.0 / 6 + t2 * (1.0 / 120 + t2 * (-1.0 / 5040 + t2 * (1.0 / 362880))));
+      eb = 0.5 + t2 * (-1.0 / 24 + t2 * (1.0 / 720 + t2 * (-1.0 / 40320 + t2 * (1.0 / 3628800))));
+      jb = 1.0 / 6 + t2 * (-1.0 / 120 + t2 * (1.0 / 5040 + t2 * (-1.0 / 362880 + t2 * (1.0 / 39916800))));
+    } else {
+      const double tt = sqrt(t2);
+      double sn, cs;
+      sincos(tt, &sn, &cs);
+      ea = sn / tt;
+      eb = (1.0 - cs) / t2;
+      jb = (tt - sn) / (t2 * tt);
+    }
+    const int r = t / 3, q = t % 3;
+    const double K = hat_e(th, t);
+    const double K2 = th[r] * th[q] - (r == q ? t2 : 0.0);
+    const double id = r == q ? 1.0 : 0.0;
+    E[t] = id + ea * K + eb * K2;
+    Jrm[t] = id - eb * K + jb * K2;
+  }
+  bar_sync<1, 128>();
+  if (t < 9) n[kNR + t] = mm_e(L, E, t, false, false);
+  else if (t >= 32 && t < 41) n[kNPhi + t - 32] = mm_e(Jrm, L + 15, t - 32, false, false);
+  bar_sync<1, 128>();
+  return n;
+}
+
+// ---- state-only terms beside the pre-integration (warps 5-7) ------------------
+
+// Jl^-1(s w), as jlinv_e with the series cut where the next term is below 1e-16.
+__device__ __forceinline__ double fast_jlinv_e(const double* w0, double s, int e) {
+  const double w[3] = {s * w0[0], s * w0[1], s * w0[2]};   // sign flips, exact
+  const double t2 = fma(w[0], w[0], fma(w[1], w[1], w[2] * w[2]));
+  const int r = e / 3, q = e - 3 * r;
+  double c;
+  if (t2 < 1e-5) {
+    c = fma(t2, fma(t2, 1.0 / 30240, 1.0 / 720), 1.0 / 12);
+  } else if (t2 < kSeriesT2) {
+    c = 1.0 / 12 + t2 * (1.0 / 720 + t2 * (1.0 / 30240 + t2 * (1.0 / 1209600 + t2 * (1.0 / 47900160))));
+  } else {
+    const double t = sqrt(t2);
+    double sn, co;
+    sincos(t, &sn, &co);
+    c = 1.0 / t2 - (1.0 + co) / (2.0 * t * sn);
+  }
+  return fma(c, fma(w[r], w[q], r == q ? -t2 : 0.0), fma(-0.5, hat_e(w, e), r == q ? 1.0 : 0.0));
+}
+
+// Rotations of the states and everything that needs them only; warp 5.
+__device__ void fast_state_terms(const SolveParams& sp, FastSmem& S) {
+  const int lane = threadIdx.x & 31, g3 = lane / 9, e9 = lane - 9 * g3;
+  const double T = S.el[kElT];
+  const double* Rc = sp.R_CS;
+  if (lane < 27) (g3 == 0 ? S.R0 : g3 == 1 ? S.Q0 : S.R1)[e9] =
+      quat_rot_e(g3 == 0 ? S.x0.q : g3 == 1 ? S.x0.qg : S.x1.q, e9);
+  else if (lane < 30) S.c[lane - 27] = fma(S.x0.v[lane - 27], T, lane == 29 ? -0.5 * sp.g * T * T : 0.0);
+  __syncwarp();
+  if (lane < 27) (g3 == 0 ? S.A0 : g3 == 1 ? S.QR : S.RcR1T)[e9] =
+      mm_e(g3 == 0 ? S.R0 : g3 == 1 ? S.Q0 : Rc, g3 == 0 ? Rc : g3 == 1 ? S.R0 : S.R1, e9, g3 == 2, g3 == 2);
+  else if (lane < 30) S.dr[lane - 27] = S.x1.r[lane - 27] - S.x0.r[lane - 27];
+  __syncwarp();
+  if (lane < 9) {
+    S.QA[lane] = mm_e(S.QR, Rc, lane, false, false);
+  } else if (lane < 18) {
+    const int k = (lane - 9) / 3, i = (lane - 9) % 3;
+    const double* A = k == 0 ? S.R0 : k == 1 ? S.Q0 : Rc;
+    const double* x = k == 1 ? S.c : sp.r_CS;
+    (k == 0 ? S.t1 : k == 1 ? S.t2c : S.rcS)[i] = mv_e(A, x, i, k != 0);
+  } else if (lane < 27) {
+    S.Jyr[e9 / 3][e9 % 3] = T * S.Q0[3 * (e9 % 3) + e9 / 3];          // position by velocity: T Q0^T
+  }
+  __syncwarp();
+  double hr = 0.0;
+  if (lane < 9) {                    // position by gravity: Q0^T [c]x, first two columns
+    const double v = mhat_e(S.Q0, true, S.c, lane);
+    if (lane % 3 < 2) S.Jyr[lane / 3][9 + lane % 3] = v;
+  } else if (lane < 18) {
+    hr = hatm_e(S.dr, S.R0, e9);     // [r1 - r0]x R0
+  } else if (lane < 21) {
+    const int i = lane - 18;
+    S.base[i] = ((S.x0.r[i] + S.t1[i]) + S.t2c[i]) - S.x1.r[i];
+  } else if (lane < 27) {
+    const int i = lane - 21;
+    S.eb[i] = i < 3 ? S.x0.bg[i] - S.x1.bg[i] : S.x0.ba[i - 3] - S.x1.ba[i - 3];
+  }
+  // C: the photometric local Jacobian on p0, -[R0 0; [dr]x R0, R0], and on p1,
+  // diag(R0, R0); the ICP one on p1, diag(R_ref, R_ref)
+  for (int idx = lane; idx < 108; idx += 32) {
+    const int i = idx / 6, k = idx - 6 * i, b = i / 3, r = i - 3 * b, kb = k / 3, q = k - 3 * kb;
+    double v = 0.0;
+    if ((b & 1) == kb) v = b < 2 ? -S.R0[3 * r + q] : b < 4 ? S.R0[3 * r + q] : S.Rref[3 * r + q];
+    if (!(b == 1 && kb == 0)) S.C[i][k] = v;
+  }
+  if (lane >= 9 && lane < 18) S.C[3 + e9 / 3][e9 % 3] = -hr;
+  __syncwarp();
+}
+
+// x1's gravity in closed form; warp 6.  e_g = log(Q0 Q1^T), its Jacobians
+// A = Jl^-1 (x0) and B = -Jr^-1 (x1), two columns each; n the unit normal of B's
+// range: the remaining row is a = A^T n with value s = n . e_g, and
+// dg1 = -Gm (e_g + A dg0) with Gm = (B^T B)^-1 B^T.
+__device__ void fast_gravity(FastSmem& S, bool gyro) {
+  const int lane = threadIdx.x & 31;
+  {
+    const int k = lane & 3;
+    const double a[4] = {S.x0.qg[0], S.x0.qg[1], S.x0.qg[2], S.x0.qg[3]};
+    double o = quat_mul_k(a, S.x1.qg, k, true);
+    const double w = __shfl_sync(0xffffffffu, o, lane & ~3);
+    if (w < 0.0) o = -o;
+    double s2 = k ? o * o : 0.0;
+    s2 += __shfl_xor_sync(0xffffffffu, s2, 1);
+    s2 += __shfl_xor_sync(0xffffffffu, s2, 2);
+    const double f = quat_log_factor(s2, fabs(w));
+    if (lane > 0 && lane < 4) S.eg[lane - 1] = f * o;
+  }
+  __syncwarp();
+  if (lane < 18) (lane < 9 ? S.Jlg : S.Jrg)[lane % 9] = fast_jlinv_e(S.eg, lane < 9 ? 1.0 : -1.0, lane % 9);
+  __syncwarp();
+  const double* B = S.Jrg;           // B = -Jrg; column m of row k at 3 k + m
+  if (lane < 3) {                    // cross product of B's columns (the signs cancel)
+    const int i1 = lane == 2 ? 0 : lane + 1, i2 = lane == 0 ? 2 : lane - 1;
+    S.nv[lane] = fma(B[3 * i1], B[3 * i2 + 1], -(B[3 * i2] * B[3 * i1 + 1]));
+  } else if (lane < 6) {             // m00, m01, m11
+    const int p = lane == 5 ? 1 : 0, q = lane == 3 ? 0 : 1;
+    S.mm[lane - 3] = fma(B[p], B[q], fma(B[3 + p], B[3 + q], B[6 + p] * B[6 + q]));
+  } else if (lane < 12) {
+    S.Ag[lane - 6] = S.Jlg[3 * ((lane - 6) >> 1) + ((lane - 6) & 1)];
+  }
+  __syncwarp();
+  const double n2 = fma(S.nv[0], S.nv[0], fma(S.nv[1], S.nv[1], S.nv[2] * S.nv[2]));
+  const double inv = rsqrt(n2);
+  if (lane < 3) {
+    double v = 0.0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) v = fma(S.nv[k], lane < 2 ? S.Jlg[3 * k + lane] : S.eg[k], v);
+    v = gyro ? 0.0 : v * inv;
+    if (lane < 2) S.a[lane] = v;
+    else S.s = v;
+  } else if (lane < 9) {             // Gm row m, column k; det(B^T B) = |n|^2 (Lagrange's identity)
+    const int m = (lane - 3) / 3, k = (lane - 3) % 3;
+    const double det = fma(S.mm[0], S.mm[2], -(S.mm[1] * S.mm[1]));
+    const double b0 = -B[3 * k], b1 = -B[3 * k + 1];
+    const double v = m == 0 ? fma(S.mm[2], b0, -(S.mm[1] * b1)) : fma(S.mm[0], b1, -(S.mm[1] * b0));
+    S.Gm[3 * m + k] = gyro ? 0.0 : v / det;
+  }
+  __syncwarp();
+}
+
+// Prior at x0: d = x0 boxminus xbar, the mean m = P b_y - d_y + K d_p of y and the
+// prior vector b_p' - H_pp' d_p on p0; warp 7.  d_v, d_ba, d_g are held in the
+// gyro-only variant.
+__device__ void fast_prior(FastSmem& S, bool gyro) {
+  const int lane = threadIdx.x & 31;
+  warp_state_boxminus(S.x0, S.xbar, S.d);
+  const double* K = S.el + kElK;
+  const double* Hp = S.el + kElHp;
+  if (lane < 17) {
+    const bool y = lane < 11;
+    const int i = y ? lane : lane - 11;
+    double v = y ? S.el[kElM0 + i] - S.d[6 + i] : S.el[kElBp + i];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) v = fma(y ? K[6 * i + k] : -Hp[6 * i + k], S.d[k], v);
+    if (y && gyro && (i < 3 || i >= 6)) v = 0.0;
+    (y ? S.m : S.bp)[i] = v;
+  }
+  __syncwarp();
+}
+
+// ---- the pixel terms (warps 4-7) ------------------------------------------------
+
+// P12 (lower triangle) and g12: U = w C H_loc for both terms, then U C^T.
+__device__ void fast_pixel_terms(const SolveParams& sp, const Ctrl* c, FastSmem& S) {
+  const int t = threadIdx.x - 128;
+  if (t < kSumsAll) S.sums[t] = __ldcg(c->sums + t);
+  bar_sync<3, 128>();
+  if (t < 126) {
+    const int i = t / 7, q = t - 7 * i;
+    const bool icp = i >= 12;
+    const double* s = S.sums + (icp ? 0 : kSums);
+    const double w = icp ? sp.W_icp : sp.W_rgb;
+    double v = 0.0;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      const int lo = min(k, q), hi = max(k, q);
+      const double h = q == 6 ? s[21 + k] : s[lo * 6 - lo * (lo - 1) / 2 + (hi - lo)];
+      v = fma(S.C[i][k], h, v);
+    }
+    S.U[i][q] = w * v;
+  }
+  bar_sync<3, 128>();
+  if (t < 78) {
+    int i = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
+    while (tri(i + 1, 0) <= t) ++i;
+    while (tri(i, 0) > t) --i;
+    const int j = t - tri(i, 0);
+    double v = 0.0;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) v = fma(S.U[i][k], S.C[j][k], v);
+    if (j >= 6) {                    // the block-diagonal ICP map: three columns of a row
+      const int b = j < 9 ? 0 : 3;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) v = fma(S.U[i + 6][b + k], S.C[j + 6][b + k], v);
+    }
+    S.P12[i * kPose + j] = v;
+  } else if (t >= 96 && t < 96 + kPose) {
+    const int i = t - 96;
+    S.g12[i] = i < 6 ? -S.U[i][6] : -(S.U[i][6] + S.U[i + 6][6]);
+  }
+}
+
+// ---- the sweep ---------------------------------------------------------------------
+
+// 1 / |d| as pivot_recip, sign restored.
+__device__ __forceinline__ double signed_recip(double d, bool neg) {
+  const double r = pivot_recip(neg ? -d : d);
+  return neg ? -r : r;
+}
+
+// One Gauss-Newton step (every thread of the block); status and all that is
+// uniform has been checked by the caller.
+__device__ void gn_step_fast(const SolveParams& sp, Ctrl* c, FastSmem& S) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const bool gyro = sp.track_mode == DRI_TRACK_GYRO_ONLY;
+  {                                   // one round of independent loads
+    const double* e = c->elim.m;
+    for (int i = tid; i < kElimDoubles; i += kSolveThreads) S.el[i] = e[i];
+    const double* p = &c->elim.piece[0][0];
+    double* q = &S.piece[0][0];
+#pragma unroll
+    for (int i = 0; i < kElimPieces * 8 / kSolveThreads; ++i) q[tid + i * kSolveThreads] = p[tid + i * kSolveThreads];
+    if (tid < 20) reinterpret_cast<double*>(&S.x0)[tid] = reinterpret_cast<const double*>(&c->x0)[tid];
+    else if (tid < 40) reinterpret_cast<double*>(&S.x1)[tid - 20] = reinterpret_cast<const double*>(&c->x1)[tid - 20];
+    else if (tid < 60) reinterpret_cast<double*>(&S.xbar)[tid - 40] = reinterpret_cast<const double*>(&c->xbar)[tid - 40];
+    else if (tid >= 64 && tid < 73) S.Rref[tid - 64] = c->Rref[tid - 64];
+  }
+  const int np = c->elim.np;
+  __syncthreads();
+  const double* root = nullptr;
+  if (warp < 4) {
+    if (sp.imu_mode == DRI_IMU_FIRST_ORDER) {
+      root = fast_first_order(sp, c, S, np);
+    } else {
+      fast_leaves(S, np, S.x0.bg, S.x0.ba);
+      root = fast_tree(S, np);
+    }
+  } else if (warp == 5) {
+    fast_state_terms(sp, S);
+  } else if (warp == 6) {
+    fast_gravity(S, gyro);
+  } else if (warp == 7) {
+    fast_prior(S, gyro);
+  }
+  __syncthreads();
+  const double* Py = S.el + kElPy;
+  const double* K = S.el + kElK;
+  if (warp >= 4) {                    // the pixel kernel's sums
+    grid_dep_wait();
+    fast_pixel_terms(sp, c, S);
+    bar_arrive<4, 256>();             // P12, g12 to the sweep
+    if (warp == 7) {                  // IMU cost at this linearisation: e^T W e
+      bar_sync<7, 160>();             // the errors (warps 0-3)
+      double v = 0.0;
+      if (lane < 18) {
+        auto err = [&](int i) {
+          return i < 3 ? S.er[i] : i < 6 ? S.ea[i - 3] : i < 9 ? S.ev[i - 6] : i < 15 ? S.eb[i - 9] : S.eg[i - 15];
+        };
+        const double* W = c->Wimu + lane * 18;
+        if (lane < 9) {
+          for (int k = 0; k < 9; ++k) v = fma(W[k], err(k), v);
+          v *= err(lane);
+        } else {
+          v = W[lane] * err(lane) * err(lane);
+        }
+      }
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (lane == 0) S.cost = v;
+    }
+  } else {
+    // ---- IMU rows ----
+    if (warp == 0) {
+      const int g3 = lane / 9, e9 = lane - 9 * g3;
+      if (lane < 9) {
+        S.RW[lane] = mm_e(S.A0, root + kNR, lane, false, false);
+      } else if (lane < 18) {         // position by b_a
+        S.Jyr[e9 / 3][6 + e9 % 3] = mm_e(S.A0, root + kNPa, e9, false, false);
+      } else if (lane < 27) {
+        S.APg[e9] = mm_e(S.A0, root + kNP, e9, false, false);
+      } else if (lane < 30) {
+        S.t3[lane - 27] = mv_e(S.A0, root + kNp, lane - 27, false);
+      }
+      __syncwarp();
+      if (lane < 9) S.M[lane] = mm_e(S.RW, S.RcR1T, lane, false, false);
+      else if (lane < 18) S.RP[e9] = mm_e(S.RW, root + kNPhi, e9, false, false);
+      else if (lane < 21) S.t4[lane - 18] = mv_e(S.RW, S.rcS, lane - 18, false);
+      __syncwarp();
+      if (lane < 9) {                 // position by b_g
+        const double v = S.APg[lane] + hatm_e(S.t4, S.RP, lane);
+        S.Jyr[lane / 3][3 + lane % 3] = v;
+      } else if (lane < 12) {
+        const int i = lane - 9;
+        S.er[i] = (S.base[i] + S.t3[i]) - S.t4[i];
+      } else if (lane < 15) {
+        const int i = lane - 12;
+        S.u[i] = (S.t1[i] + S.t3[i]) - S.t4[i];
+      }
+      __syncwarp();
+      if (gyro) {                     // the position rows carry no weight: no information
+        for (int i = lane; i < 33; i += 32) S.Jyr[i / 11][i % 11] = 0.0;
+        __syncwarp();
+      }
+      bar_arrive<5, 96>();
+      // e_a = log(M): the skew part v = 2 sin(t) k, t / (2 sin t) from its series in
+      // sin^2 t (the angle is below 6.4 mrad in all but a frame's first iterations)
+      double ea;
+      {
+        const int i = lane % 3, i1 = i == 2 ? 0 : i + 1, i2 = i == 0 ? 2 : i - 1;
+        const double v = 0.5 * (S.M[3 * i2 + i1] - S.M[3 * i1 + i2]);
+        const double v0 = __shfl_sync(0xffffffffu, v, 0), v1 = __shfl_sync(0xffffffffu, v, 1),
+                     v2 = __shfl_sync(0xffffffffu, v, 2);
+        const double s2 = fma(v0, v0, fma(v1, v1, v2 * v2));
+        const float tr = (float)S.M[0] + (float)S.M[4] + (float)S.M[8];
+        if (s2 < 4e-5 && tr > 2.f) ea = v * fma(s2, fma(s2, fma(s2, 5.0 / 112, 3.0 / 40), 1.0 / 6), 1.0);
+        else ea = log_i(S.M, i);
+      }
+      if (lane < 3) S.ea[lane] = ea;
+      __syncwarp();
+      if (lane < 18) (lane < 9 ? S.Jla : S.Jra)[e9] = fast_jlinv_e(S.ea, lane < 9 ? 1.0 : -1.0, e9);
+      __syncwarp();
+      if (lane < 9) S.B13[lane] = mm_e(S.Jla, S.RP, lane, false, false);
+    } else if (warp == 3) {           // velocity rows, used for dv1 only
+      if (lane < 9) S.B14[lane] = mm_e(S.QA, root + kNV, lane, false, false);
+      else if (lane < 18) S.B17[lane - 9] = mm_e(S.QA, root + kNVa, lane - 9, false, false);
+      else if (lane < 24) {
+        const int k = (lane - 18) / 3, i = (lane - 18) % 3;
+        (k == 0 ? S.w9 : S.t5)[i] = mv_e(k == 0 ? S.A0 : S.QA, root + kNv, i, false);
+      }
+      __syncwarp();
+      if (lane < 9) S.B9[lane] = -mhat_e(S.Q0, false, S.w9, lane);
+      else if (lane < 18) {
+        const int e = lane - 9;
+        if (e % 3 < 2) S.B20[2 * (e / 3) + e % 3] = -hat_e(S.t5, e);
+      } else if (lane < 21) {
+        const int i = lane - 18;
+        S.ev[i] = (fma(i == 2 ? -sp.g : 0.0, S.el[kElT], S.x0.v[i]) + S.t5[i]) - S.x1.v[i];
+      }
+    }
+    if (warp == 1 || warp == 2) {     // position rows: Jy P, Jp + Jy K, e + Jy m
+      bar_sync<5, 96>();
+      const int q = lane - 11;
+      const int r = warp == 1 ? lane / 11 : lane < 11 ? 2 : lane < 29 ? q / 6 : lane - 29;
+      const int cc = warp == 1 ? lane - 11 * r : lane < 11 ? lane : lane < 29 ? q - 6 * r : 0;
+      const double* B = (warp == 1 || lane < 11) ? Py + cc : lane < 29 ? K + cc : S.m;
+      const int sb = (warp == 1 || lane < 11) ? 11 : lane < 29 ? 6 : 1;
+      if (warp == 2 || lane < 22) {
+        double v = 0.0;
+        if (warp == 2 && lane >= 29) v = gyro ? 0.0 : S.er[r];
+        else if (warp == 2 && lane >= 11 && !gyro) v = cc < 3 ? (cc == r ? 1.0 : 0.0) : -hat_e(S.u, 3 * r + cc - 3);
+#pragma unroll
+        for (int k = 0; k < 11; ++k) v = fma(S.Jyr[r][k], B[k * sb], v);
+        if (warp == 1 || lane < 11) S.T[r][cc] = v;
+        else if (lane < 29) S.Jp[r][cc] = v;
+        else S.ep[r] = v;
+      }
+      bar_sync<6, 64>();
+      if (warp == 1 && lane < 6) {
+        const int i = lane < 1 ? 0 : lane < 3 ? 1 : 2, j = lane - tri(i, 0);
+        double v = 0.0;
+#pragma unroll
+        for (int k = 0; k < 11; ++k) v = fma(S.T[i][k], S.Jyr[j][k], v);
+        S.S[tri(i, j)] = v;
+      }
+    }
+    if (warp < 3) {
+      bar_sync<5, 96>();
+      // rotation rows (their only y column block is b_g: B13) and the gravity row
+      if (warp == 0) {
+        if (lane < 9) {
+          const int i = lane / 3, j = lane - 3 * i;
+          double v = 0.0;
+#pragma unroll
+          for (int k = 0; k < 3; ++k) v = fma(S.B13[3 * i + k], S.T[j][3 + k], v);
+          S.S[tri(3 + i, j)] = v;
+        } else if (lane < 20) {
+          const int q = lane - 9;
+          S.T[6][q] = fma(S.a[0], Py[9 * 11 + q], S.a[1] * Py[10 * 11 + q]);
+        } else if (lane < 23) {
+          const int j = lane - 20;
+          S.S[tri(6, j)] = fma(S.a[0], S.T[j][9], S.a[1] * S.T[j][10]);
+        } else if (lane < 29) {
+          const int q = lane - 23;
+          S.Jp[6][q] = fma(S.a[0], K[9 * 6 + q], S.a[1] * K[10 * 6 + q]);
+        } else if (lane == 29) {
+          S.ep[6] = S.s + fma(S.a[0], S.m[9], S.a[1] * S.m[10]);
+        }
+      } else {
+        const int q = lane - 11;
+        const int r = warp == 1 ? lane / 11 : lane < 11 ? 2 : lane < 29 ? q / 6 : lane - 29;
+        const int cc = warp == 1 ? lane - 11 * r : lane < 11 ? lane : lane < 29 ? q - 6 * r : 0;
+        const double* B = (warp == 1 || lane < 11) ? Py + 33 + cc : lane < 29 ? K + 18 + cc : S.m + 3;
+        const int sb = (warp == 1 || lane < 11) ? 11 : lane < 29 ? 6 : 1;
+        if (warp == 2 || lane < 22) {
+          double v = 0.0;
+          if (warp == 2 && lane >= 29) v = S.ea[r];
+          else if (warp == 2 && lane >= 11 && cc >= 3) v = S.Jla[3 * r + cc - 3];
+#pragma unroll
+          for (int k = 0; k < 3; ++k) v = fma(S.B13[3 * r + k], B[k * sb], v);
+          if (warp == 1 || lane < 11) S.T[3 + r][cc] = v;
+          else if (lane < 29) S.Jp[3 + r][cc] = v;
+          else S.ep[3 + r] = v;
+        }
+      }
+      // the rows' constant parts on p1: -I, -Jr^-1
+      if (warp == 0)
+        for (int idx = lane; idx < 42; idx += 32) {
+          const int i = idx / 6, k = idx - 6 * i;
+          double v = 0.0;
+          if (i < 3) v = k == i && !gyro ? -1.0 : 0.0;
+          else if (i < 6 && k >= 3) v = -S.Jra[3 * (i - 3) + k - 3];
+          S.Jp[i][6 + k] = v;
+        }
+      bar_sync<5, 96>();
+      if (warp == 1) {
+        if (lane < 6) {
+          const int i = lane < 1 ? 0 : lane < 3 ? 1 : 2, j = lane - tri(i, 0);
+          double v = 0.0;
+#pragma unroll
+          for (int k = 0; k < 3; ++k) v = fma(S.T[3 + i][3 + k], S.B13[3 * j + k], v);
+          S.S[tri(3 + i, 3 + j)] = v;
+        } else if (lane < 10) {       // gravity row against the rotation rows and itself
+          const int j = lane - 3;     // 3, 4, 5, 6
+          S.S[tri(6, j)] = fma(S.a[0], S.T[j][9], S.a[1] * S.T[j][10]);
+        }
+      }
+    }
+    bar_arrive<7, 160>();
+    bar_sync<1, 128>();
+    // ---- the sweep: entry e of the lower triangle and the right-hand side row,
+    // longest-updated first, 32-entry chunks dealt to the four warps in turn, so
+    // that the entries a pivot still updates take the fewest warp instructions ----
+    int ei[2], ej[2];
+    double v[2];
+#pragma unroll
+    for (int o = 0; o < 2; ++o) {
+      const int e = tid + 128 * o;
+      int i = -1, j = -1;
+      double x = 0.0;
+      if (e < kSysEnt) {              // column j = 18 - g holds rows j .. 19 (19: right-hand side): g + 2 entries
+        int g = (int)((sqrtf(9.0f + 8.0f * e) - 3.0f) * 0.5f);
+        while (g * (g + 3) / 2 > e) --g;
+        while ((g + 1) * (g + 4) / 2 <= e) ++g;
+        j = kSys - 1 - g;
+        i = j + e - g * (g + 3) / 2;
+        if (i < kLam) {               // -(S + blockdiag(S6, sigma_g^2))
+          const double s6 = i < 6 ? S.el[kElS6 + 6 * i + j] : i == j ? S.el[kElSg] : 0.0;
+          x = -(S.S[tri(i, j)] + s6);
+        } else if (j < kLam) {
+          x = i == kSys ? -S.ep[j] : S.Jp[j][i - kLam];
+        } else if (i == kSys) {
+          x = j < kLam + 6 ? S.bp[j - kLam] : 0.0;
+        } else {
+          x = i < kLam + 6 ? S.el[kElHp + 6 * (i - kLam) + j - kLam] : 0.0;
+        }
+      }
+      ei[o] = i;
+      ej[o] = j;
+      v[o] = x;
+    }
+    for (int k = 0; k < kSys; ++k) {
+      if (k == kLam) {                // the pixel terms join the pose block
+        grid_dep_wait();
+        bar_sync<4, 256>();
+#pragma unroll
+        for (int o = 0; o < 2; ++o) {
+          const int i = ei[o], j = ej[o];
+          if (j >= kLam) v[o] += i == kSys ? S.g12[j - kLam] : S.P12[(i - kLam) * kPose + j - kLam];
+        }
+      }
+      double* cb = S.col[k & 1];
+#pragma unroll
+      for (int o = 0; o < 2; ++o)
+        if (ej[o] == k) cb[ei[o]] = v[o];
+      bar_sync<1, 128>();
+      const double d = cb[k];
+      const double r = signed_recip(d, k < kLam);
+      if (tid == 0) {
+        S.piv[k] = k < kLam ? -d : d;
+        S.rinv[k] = r;
+      }
+#pragma unroll
+      for (int o = 0; o < 2; ++o)
+        if (ej[o] > k) v[o] = fma(-(cb[ei[o]] * r), cb[ej[o]], v[o]);
+    }
+    bar_sync<1, 128>();
+#pragma unroll
+    for (int o = 0; o < 2; ++o)       // unit-lower L; its row 19 holds z_k / d_k
+      if (ei[o] > ej[o]) S.L[ej[o]][ei[o]] = v[o] * S.rinv[ej[o]];
+    bar_sync<1, 128>();
+    if (warp < 2) {
+      double* dx = S.dx;
+      if (warp == 0) {
+        double y = lane < kSys ? S.L[lane][kSys] : 0.0;
+        for (int k = kSys - 1; k > 0; --k) {
+          const double xk = __shfl_sync(0xffffffffu, y, k);
+          if (lane < k) y = fma(-S.L[lane][k], xk, y);
+        }
+        if (lane < kSys) S.z[lane] = y;
+        if (lane >= kLam && lane < kSys) dx[lane < kLam + 6 ? lane - kLam : 4 + lane] = y;   // p0 at 0..5, p1 at 17..22
+        bool ok = lane >= kSys || (S.piv[lane] > 0.0 && S.piv[lane] < INFINITY);
+        ok = __all_sync(0xffffffffu, ok);
+        __syncwarp();
+        // y (lanes 0-10: K p0 + m, 16-26: -T^T lambda), dv1's part without y
+        // (11-13: e_v + B9 da0, 27-29: -S_v6 lambda)
+        const double* lam = S.z;
+        const double* p0 = S.z + kLam;
+        const int h = lane & 15;
+        const bool top = lane >= 16;
+        double w = 0.0;
+        if (h < 14) {
+          const double* A = h < 11 ? (top ? &S.T[0][h] : K + 6 * h) : (top ? S.el + kElSv + 6 * (h - 11) : S.B9 + 3 * (h - 11));
+          const int sa = h < 11 && top ? 11 : 1;
+          const double* B = top ? lam : (h < 11 ? p0 : p0 + 3);
+          const int n = h < 11 ? (top ? 7 : 6) : (top ? 6 : 3);
+          w = top ? 0.0 : h < 11 ? S.m[h] : S.ev[h - 11];
+#pragma unroll
+          for (int k = 0; k < 7; ++k)
+            if (k < n) w = fma(top ? -A[k * sa] : A[k * sa], B[k], w);
+        }
+        w += __shfl_down_sync(0xffffffffu, w, 16);
+        if (lane < 11) dx[6 + lane] = w;
+        else if (lane < 14) S.u[lane - 11] = w;            // dv1's part
+        __syncwarp();
+        bool fin = true;
+        if (lane < 17) fin = ((__double_as_longlong(dx[lane]) >> 52) & 0x7ff) != 0x7ff;
+        ok = __all_sync(0xffffffffu, fin) && ok;
+        if (lane == 0) S.good[0] = ok;
+      }
+      bar_sync<6, 64>();
+      if (warp == 0) {
+        warp_state_boxplus(S.x0, dx);
+      } else {
+        const double* y = dx + 6;     // v, b_g, b_a, gravity
+        double w = 0.0;
+        if (lane < 9) {               // dv1: row lane % 3, part lane / 3
+          const int i = lane % 3, q = lane / 3;
+          const double* A = q == 0 ? S.B14 + 3 * i : q == 1 ? S.B17 + 3 * i : S.B20 + 2 * i;
+          const double* B = q == 0 ? y + 3 : q == 1 ? y + 6 : y + 9;
+          w = q == 2 ? y[i] + S.u[i] : 0.0;
+#pragma unroll
+          for (int k = 0; k < 3; ++k)
+            if (k < 2 || q < 2) w = fma(A[k], B[k], w);
+        } else if (lane < 15) {       // x1's biases follow x0's
+          w = S.eb[lane - 9] + y[3 + lane - 9];
+          if (gyro && lane >= 12) w = 0.0;
+        } else if (lane < 18) {
+          const int i = lane - 15;
+          w = fma(S.Ag[2 * i], y[9], fma(S.Ag[2 * i + 1], y[10], S.eg[i]));
+        }
+        const double w1 = __shfl_down_sync(0xffffffffu, w, 3), w2 = __shfl_down_sync(0xffffffffu, w, 6);
+        const double u0 = __shfl_sync(0xffffffffu, w, 15), u1 = __shfl_sync(0xffffffffu, w, 16),
+                     u2 = __shfl_sync(0xffffffffu, w, 17);
+        if (lane < 3) dx[23 + lane] = gyro ? 0.0 : (w + w1) + w2;
+        else if (lane >= 9 && lane < 15) dx[26 + lane - 9] = w;
+        else if (lane >= 18 && lane < 20) {
+          const double* G = S.Gm + 3 * (lane - 18);
+          dx[32 + lane - 18] = -fma(G[0], u0, fma(G[1], u1, G[2] * u2));
+        }
+        __syncwarp();
+        bool fin = true;
+        if (lane < 17) fin = ((__double_as_longlong(dx[17 + lane]) >> 52) & 0x7ff) != 0x7ff;
+        fin = __all_sync(0xffffffffu, fin);
+        if (lane == 0) S.good[1] = fin;
+        warp_state_boxplus(S.x1, dx + 17);
+      }
+    }
+  }
+  __syncthreads();
+  if (!S.good[0] || !S.good[1]) {
+    if (tid == 0) c->status = DRI_ELOST;
+    return;
+  }
+  if (warp == 0) {
+    warp_write_transforms(c, S.x0, S.x1, S.rot);
+  } else if (warp == 1) {
+    if (lane < 20) reinterpret_cast<double*>(&c->x0)[lane] = reinterpret_cast<const double*>(&S.x0)[lane];
+  } else if (warp == 2) {
+    if (lane < 20) reinterpret_cast<double*>(&c->x1)[lane] = reinterpret_cast<const double*>(&S.x1)[lane];
+  } else if (tid == 96) {
+    c->n_icp[sp.level] = (int32_t)S.sums[28];
+    c->n_rgb[sp.level] = (int32_t)S.sums[kSums + 28];
+    store_margin(c, sp.level);
+    c->cost = sp.W_icp * S.sums[27] + sp.W_rgb * S.sums[kSums + 27] + S.cost;
+    c->iterations += 1;
+  }
+}
+
+// ---- the frame's constants (k_frame_begin) -----------------------------------------
+
+// Fills Ctrl::elim for the frame: the sweep operator over y (components 6..16) of
+// the prior's augmented matrix [H* b*] leaves -P = -H_yy^-1, P H_yp = -K, P b_y and,
+// on the pose block, the Schur complement and its vector; element-parallel on the
+// lower triangle, one of its 170 entries per thread (per pivot a reciprocal, a
+// scaling and an update).  Components that the gyro-only variant holds are left
+// out (zero rows and columns).  pk, dt: the frame's np pieces; Sg: the 9 x 9
+// covariance of the (r, a, v) rows.  Whole block.  elim.ok stays 0 when H_yy is
+// not safely positive definite or there are more pieces than the step keeps in
+// shared memory: the frame's steps then all take the information form.
+__device__ void prepare_elim(const SolveParams& sp, Ctrl* c, int np, const double* dt, const int* pk,
+                             double T, const double* Sg, double* col, int* bad) {
+  const int tid = threadIdx.x;
+  const bool gyro = sp.track_mode == DRI_TRACK_GYRO_ONLY;
+  int i = -1, j = -1;
+  double v = 0.0;
+  if (tid < 170) {                    // rows 0..16, then the row of b* (17)
+    if (tid < 153) {
+      i = (int)((sqrtf(8.f * tid + 1.f) - 1.f) * 0.5f);
+      while (tri(i + 1, 0) <= tid) ++i;
+      while (tri(i, 0) > tid) --i;
+      j = tid - tri(i, 0);
+      v = c->Hs[i * 17 + j];
+    } else {
+      i = 17;
+      j = tid - 153;
+      v = c->bs[j];
+    }
+    if (gyro && ((i < 17 && held_gyro_only(i)) || held_gyro_only(j))) v = 0.0;
+  }
+  if (tid == 0) *bad = np > kElimPieces;
+  const double diag = v;
+  double* m = c->elim.m;
+  if (np <= kElimPieces) {
+    const dri_imu_sample* s = imu_samples(sp.imu);
+    for (int L = tid; L < 8 * np; L += kSolveThreads) {
+      const int k = L >> 3, q = L & 7;
+      const dri_imu_sample& x = s[pk[k]];
+      c->elim.piece[k][q] = q == 0 ? dt[k] : q == 1 ? 0.5 * dt[k] : q < 5 ? x.gyr[q - 2] : x.acc[q - 5];
+    }
+  }
+  for (int e = tid; e < 54; e += kSolveThreads) {
+    if (e < 36) m[kElS6 + e] = Sg[(e / 6) * 9 + e % 6];
+    else m[kElSv + e - 36] = Sg[(6 + (e - 36) / 6) * 9 + (e - 36) % 6];
+  }
+  if (tid == 0) {
+    m[kElSg] = sp.sigma_grav * sp.sigma_grav;
+    m[kElT] = T;
+  }
+  __syncthreads();
+  for (int k = 6; k < 17; ++k) {
+    if (gyro && held_gyro_only(k)) continue;
+    double* ck = col + (k & 1) * 18;  // column k by symmetry
+    if (i == k) ck[j] = v;
+    else if (j == k) ck[i] = v;
+    if (i == k && j == k && !(v > 1e-12 * diag && v < 1e300)) *bad = 1;
+    __syncthreads();
+    const double r = pivot_recip(ck[k]);
+    if (i >= 0) {
+      if (i == k && j == k) v = -r;
+      else if (i == k || j == k) v = v * r;
+      else v = fma(-(ck[i] * r), ck[j], v);
+    }
+  }
+  if (i == 17) {
+    m[j < 6 ? kElBp + j : kElM0 + j - 6] = v;
+  } else if (i >= 6 && j >= 6) {
+    m[kElPy + (i - 6) * 11 + j - 6] = -v;
+    m[kElPy + (j - 6) * 11 + i - 6] = -v;
+  } else if (i >= 6) {
+    m[kElK + (i - 6) * 6 + j] = -v;
+  } else if (i >= 0) {
+    m[kElHp + i * 6 + j] = v;
+    m[kElHp + j * 6 + i] = v;
+  }
+  if (tid == 0) {
+    c->elim.np = np;
+    c->elim.ok = !*bad;
+  }
+}

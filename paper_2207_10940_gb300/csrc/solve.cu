@@ -2,8 +2,10 @@
 //
 //   frame_begin   x0 := x; IMU pre-integration at x0's biases with the propagated
 //                 noise covariance; W_IMU = Sigma^-1; x1 := the IMU prediction x^1(x0)
-//   gn_step       one Gauss-Newton iteration: re-integrate the IMU at x0's current
-//                 biases, IMU error (Eq. 5) and its analytic 18x34 Jacobian; rotate
+//   gn_step       one Gauss-Newton iteration, in one of two forms: the covariance
+//                 form (joint_step.cuh) for all but a frame's last one, and the
+//                 information form below, which also leaves the full system for
+//                 the marginalisation: re-integrate the IMU at x0's current biases, IMU error (Eq. 5) and its analytic 18x34 Jacobian; rotate
 //                 the pixel kernel's photometric / ICP systems into W and map the
 //                 photometric one onto both poses; add the prior (Eq. 6/9); solve the
 //                 34x34 system of Eq. 7; x0, x1 boxplus= dx (Eq. 2)
@@ -1018,6 +1020,8 @@ __device__ __forceinline__ void store_margin(Ctrl* c, int level) {
   c->margin_acc[0] = c->margin_acc[1] = 0u;
 }
 
+#include "joint_step.cuh"
+
 // Assemble the joint system at (ctrl->x0, ctrl->x1) into S.H (full), S.b.
 // Entry e (0..71) of the two pixel systems rotated into W: term e / 36 (0 ICP
 // with R_ref, 1 photometric with R_0), element e % 36 of its 6x6 (and, for
@@ -1654,6 +1658,7 @@ struct BeginSmem {
   ImuLin L;
   double G[81], GS[81], Sg[81], Winv[81];
   double col[18];
+  double ecol[36];
   double rot[18];
   int ok, fail;
 };
@@ -1721,6 +1726,10 @@ __device__ bool imu_weight_and_prediction(const SolveParams& sp, Ctrl* c, BeginS
   __syncthreads();
   if (tid < 81) B.Sg[tid] = sym;
   __syncthreads();
+  if (sp.gdof != 3) {                 // the steps' constants (joint_step.cuh)
+    prepare_elim(sp, c, B.W.np, B.W.dt, B.W.pk, B.P.T, B.Sg, B.ecol, &B.fail);
+    __syncthreads();
+  }
   const bool pd = block_ldlt(B.Sg, 9, 9, B.col, &B.fail);
   if (tid < 9) {
     double colv[9];
@@ -1983,16 +1992,28 @@ __global__ void __launch_bounds__(kSolveThreads) k_frame_begin_batch(const Batch
   if (load_slot_params(a, sp) == kSlotTrack) frame_begin_body(sp, *reinterpret_cast<BeginSmem*>(smem_raw));
 }
 
-constexpr size_t kGnSmemMax = sizeof(Gn3Smem) > sizeof(GnSmem) ? sizeof(Gn3Smem) : sizeof(GnSmem);
+constexpr size_t kGnSmem2 = sizeof(FastSmem) > sizeof(GnSmem) ? sizeof(FastSmem) : sizeof(GnSmem);
+constexpr size_t kGnSmemMax = sizeof(Gn3Smem) > kGnSmem2 ? sizeof(Gn3Smem) : kGnSmem2;
 
-__global__ void __launch_bounds__(kSolveThreads) k_gn_step_batch(const BatchArgs a) {
+__global__ void __launch_bounds__(kSolveThreads, 1) k_gn_step_batch(const BatchArgs a) {
   __shared__ SolveParams sp;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   grid_dep_launch();                    // the next pixel kernel waits for this step itself
   const int mode = load_slot_params(a, sp);
-  if (mode == kSlotTrack && sp.gdof == 3) gn_step_g3(sp, *reinterpret_cast<Gn3Smem*>(smem_raw));
-  else if (mode == kSlotTrack) gn_step_body(sp, *reinterpret_cast<GnSmem*>(smem_raw));
-  else grid_dep_wait();                 // idle slot: nothing to read, keep the ordering
+  if (mode == kSlotTrack && sp.gdof == 3) {
+    gn_step_g3(sp, *reinterpret_cast<Gn3Smem*>(smem_raw));
+  } else if (mode == kSlotTrack) {
+    // the covariance form, except where the full system is wanted (marginalisation
+    // after the last iteration) or the frame's prior does not allow it
+    Ctrl* c = sp.ctrl;
+    if (!sp.last && sp.track_mode != DRI_TRACK_RGBD_ONLY && c->elim.ok) {
+      if (c->status == 0) gn_step_fast(sp, c, *reinterpret_cast<FastSmem*>(smem_raw));
+    } else {
+      gn_step_body(sp, *reinterpret_cast<GnSmem*>(smem_raw));
+    }
+  } else {
+    grid_dep_wait();                    // idle slot: nothing to read, keep the ordering
+  }
 }
 
 // A first frame is initialised here too, so that the map sets of every slot
@@ -2060,7 +2081,7 @@ cudaError_t launch_gn_step_batch(const BatchArgs& a, bool g3, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(a.nslots);
   cfg.blockDim = dim3(kSolveThreads);
-  cfg.dynamicSmemBytes = g3 ? kGnSmemMax : sizeof(GnSmem);
+  cfg.dynamicSmemBytes = g3 ? kGnSmemMax : kGnSmem2;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
