@@ -31,9 +31,11 @@
 // This is the same minimiser as Eq. 7's in exact arithmetic; the 1e8-scale IMU
 // weights are never formed (their inverses are added instead).
 //
-// Measured against the information form (`gn_step_body`): a step on one block 102k ->
-// 66k cycles, one 640x480 camera 1207 -> 914 us per frame, 12 x 320x240 1471 -> 1110
-// us, 64 x 640x480 (steps hidden behind other groups' pixels) 4710 -> 4621 us.
+// Measured against the information form (`gn_step_body`): a step on one block 102k
+// -> 46k cycles (66k with the same algebra but branches between the lanes of a
+// phase, index arithmetic per element and FP64 comparisons); one 640x480 camera
+// 1201 -> 743 us per frame, 12 x 320x240 1449 -> 935 us, 64 x 640x480 (steps hidden
+// behind other groups' pixels) 4734 -> 4547 us.
 //
 // Included by solve.cu, inside its namespace, after the element-wise 3x3 algebra
 // and the warp-cooperative state algebra that it uses.
@@ -60,17 +62,18 @@ struct FastSmem {
   double piece[kElimPieces][8];       // as Elim::piece
   double el[kElimDoubles];            // Elim's matrices
   DState x0, x1, xbar;
-  double Rref[9];
+  double Rref[9], rref[3];
+  double one, zero;
   double dx[34];                      // the step
   // states only
-  double R0[9], Q0[9], R1[9], A0[9], QR[9], QA[9], RcR1T[9], c[3], t1[3], t2c[3], rcS[3], base[3], dr[3];
+  double R0[9], Q0[9], R1[9], A0[9], QR[9], QA[9], RcR1T[9], c[3], t1[3], t2c[3], rcS[3], base[3], dr[3], evb[3];
   double d[17], m[11], bp[6];         // x0 boxminus xbar; mean of y; prior vector on p0
-  double eg[3], Jlg[9], Jrg[9], nv[3], mm[3], a[2], s, Gm[6], Ag[6];
+  double eg[3], Jlg[9], Jrg[9], nv[3], mm[3], a[3], s, Gm[6], Ag[6];
   double eb[6];                       // bias errors
   double C[18][6];                    // pixel Jacobian maps: photometric on (p0, p1), ICP on p1
   // after the pre-integration
   double Jyr[3][11];                  // position rows by y
-  double RW[9], APg[9], t3[3], M[9], RP[9], t4[3], u[3], er[3], ea[3], Jla[9], Jra[9], B13[9];
+  double RW[9], APg[9], t3[3], M[9], RP[9], t4[3], u[3], er[3], ea[3], Jla[9], B13[9];
   double B14[9], B17[9], w9[3], t5[3], B9[9], B20[6], ev[3];
   double T[kLam][11];                 // Jy P
   double Jp[kLam][kPose];             // J'
@@ -82,73 +85,105 @@ struct FastSmem {
   double P12[kPose * kPose], g12[kPose];
   // sweep
   double col[2][kSys + 1];
-  double rinv[kSys], piv[kSys], z[kSys];
+  double sink[128];                   // where a lane without a value to publish writes
+  double z[kSys];
   double L[kSys][kSys + 2];
-  double rot[18];
+  double rot[24];
   double fo[21];
   double cost;
-  int good[2];
+  int good[2], posdef[4];
+};
+template <int N>
+struct Slots {
+  static constexpr int value = N;
 };
 
 __device__ __forceinline__ int tri(int i, int j) { return i * (i + 1) / 2 + j; }   // i >= j
+
+// a < b for non-negative doubles, as integers (an FP64 comparison would take the
+// FP64 pipe for 64 cycles).
+__device__ __forceinline__ bool pos_less(double a, double b) {
+  return __double_as_longlong(a) < __double_as_longlong(b);
+}
+__device__ __forceinline__ bool finite_bits(double a) {
+  return (__double2hiint(a) & 0x7ff00000) != 0x7ff00000;
+}
+
+// base + three products along strides.  Lanes that take different products of a
+// phase differ in their pointers only: branches of a warp would run one after the
+// other, each holding the FP64 pipe for its own instructions.
+__device__ __forceinline__ double dot3(double base, const double* A, int sa, const double* B, int sb) {
+  return fma(A[0], B[0], fma(A[sa], B[sb], fma(A[2 * sa], B[2 * sb], base)));
+}
+// the same with the third product's operands given apart
+__device__ __forceinline__ double dot21(double base, const double* A, const double* B, int sb,
+                                        const double* A2, const double* B2) {
+  return fma(A[0], B[0], fma(A[1], B[sb], fma(*A2, *B2, base)));
+}
 
 // ---- IMU pieces --------------------------------------------------------------
 
 // Leaves of the pieces at biases (bg, ba): R = Exp(th), Phi = -Jr(th) dt, v = a dt,
 // p = a dt^2 / 2, Va = -dt I, Pa = -dt^2 / 2 I.  Warps 0-3.  The three series (or
-// sines) of a piece run on three lanes, its nine matrix elements on nine.
+// sines) of a piece run on three lanes, its nine matrix elements on nine; a
+// thread keeps its element and strides over the pieces, so that the index
+// arithmetic (divisions by 9 and 3) is done once.
 __device__ void fast_leaves(FastSmem& S, int np, const double* bg, const double* ba) {
-  const int t = threadIdx.x;
-  for (int L = t; L < 6 * np; L += 128) {
-    const int q = L / np, k = L - q * np;
-    const double* pc = S.piece[k];
-    if (q < 3) {
-      S.th[k][q] = (pc[2 + q] - bg[q]) * pc[0];
-    } else {
-      const double v = (pc[2 + q] - ba[q - 3]) * pc[0];
-      S.nodeA[k][kNv + q - 3] = v;
-      S.nodeA[k][kNp + q - 3] = v * pc[1];
+  const int t = threadIdx.x, q = t >> 4;
+  if (q < 6)
+    for (int k = t & 15; k < np; k += 16) {
+      const double* pc = S.piece[k];
+      if (q < 3) {
+        S.th[k][q] = (pc[2 + q] - bg[q]) * pc[0];
+      } else {
+        const double v = (pc[2 + q] - ba[q - 3]) * pc[0];
+        S.nodeA[k][kNv + q - 3] = v;
+        S.nodeA[k][kNp + q - 3] = v * pc[1];
+      }
     }
-  }
   bar_sync<1, 128>();
-  for (int L = t; L < 3 * np; L += 128) {
-    const int q = L / np, k = L - q * np;
-    const double* w = S.th[k];
-    const double t2 = fma(w[0], w[0], fma(w[1], w[1], w[2] * w[2]));
-    double f;
-    if (t2 < kSeriesT2) {            // sin t / t, (1 - cos t) / t^2, (t - sin t) / t^3
-      const double c0 = q == 0 ? 1.0 : q == 1 ? 0.5 : 1.0 / 6;
-      const double c1 = q == 0 ? -1.0 / 6 : q == 1 ? -1.0 / 24 : -1.0 / 120;
-      const double c2 = q == 0 ? 1.0 / 120 : q == 1 ? 1.0 / 720 : 1.0 / 5040;
-      const double c3 = q == 0 ? -1.0 / 5040 : q == 1 ? -1.0 / 40320 : -1.0 / 362880;
-      const double c4 = q == 0 ? 1.0 / 362880 : q == 1 ? 1.0 / 3628800 : 1.0 / 39916800;
-      f = fma(t2, fma(t2, fma(t2, fma(t2, c4, c3), c2), c1), c0);
-    } else {
-      const double th = sqrt(t2);
-      double sn, cs;
-      sincos(th, &sn, &cs);
-      f = q == 0 ? sn / th : q == 1 ? (1.0 - cs) / t2 : (th - sn) / (t2 * th);
+  if (q < 3)
+    for (int k = t & 15; k < np; k += 16) {
+      const double* w = S.th[k];
+      const double t2 = fma(w[0], w[0], fma(w[1], w[1], w[2] * w[2]));
+      double f;
+      if (pos_less(t2, kSeriesT2)) { // sin t / t, (1 - cos t) / t^2, (t - sin t) / t^3
+        const double c0 = q == 0 ? 1.0 : q == 1 ? 0.5 : 1.0 / 6;
+        const double c1 = q == 0 ? -1.0 / 6 : q == 1 ? -1.0 / 24 : -1.0 / 120;
+        const double c2 = q == 0 ? 1.0 / 120 : q == 1 ? 1.0 / 720 : 1.0 / 5040;
+        const double c3 = q == 0 ? -1.0 / 5040 : q == 1 ? -1.0 / 40320 : -1.0 / 362880;
+        const double c4 = q == 0 ? 1.0 / 362880 : q == 1 ? 1.0 / 3628800 : 1.0 / 39916800;
+        f = fma(t2, fma(t2, fma(t2, fma(t2, c4, c3), c2), c1), c0);
+      } else {
+        const double th = sqrt(t2);
+        double sn, cs;
+        sincos(th, &sn, &cs);
+        f = q == 0 ? sn / th : q == 1 ? (1.0 - cs) / t2 : (th - sn) / (t2 * th);
+      }
+      S.ser[q][k] = f;
+      if (q == 0) S.t2[k] = t2;
     }
-    S.ser[q][k] = f;
-    if (q == 0) S.t2[k] = t2;
-  }
   bar_sync<1, 128>();
-  for (int L = t; L < 9 * np; L += 128) {
-    const int k = L / 9, e = L - 9 * k, r = e / 3, c = e - 3 * r;
-    const double* w = S.th[k];
-    const double dt = S.piece[k][0], hdt = S.piece[k][1];
-    const double id = r == c ? 1.0 : 0.0;
-    const double K = hat_e(w, e), K2 = fma(w[r], w[c], r == c ? -S.t2[k] : 0.0);
-    const double ea = S.ser[0][k], eb = S.ser[1][k], jb = S.ser[2][k];
-    double* n = S.nodeA[k];
-    n[kNR + e] = fma(eb, K2, fma(ea, K, id));
-    n[kNPhi + e] = -dt * fma(jb, K2, fma(-eb, K, id));
-    n[kNV + e] = 0.0;
-    n[kNP + e] = 0.0;
-    n[kNVa + e] = r == c ? -dt : 0.0;
-    n[kNPa + e] = r == c ? -hdt * dt : 0.0;
-    if (e == 0) n[kNT] = dt;
-  }
+  const int k0 = t / 9, e = t - 9 * k0, r = e / 3, c = e - 3 * r;
+  const int hk = r == c ? 0 : 3 - r - c;                      // [w]x element e: +-w[hk], or 0
+  const bool neg = ((c - r + 3) % 3) == 1, diag = r == c;
+  const double id = diag ? 1.0 : 0.0;
+  if (k0 < 14)
+    for (int k = k0; k < np; k += 14) {
+      const double* w = S.th[k];
+      const double dt = S.piece[k][0], hdt = S.piece[k][1];
+      const double wk = w[hk];
+      const double K = diag ? 0.0 : neg ? -wk : wk, K2 = fma(w[r], w[c], diag ? -S.t2[k] : 0.0);
+      const double ea = S.ser[0][k], eb = S.ser[1][k], jb = S.ser[2][k];
+      double* n = S.nodeA[k];
+      n[kNR + e] = fma(eb, K2, fma(ea, K, id));
+      n[kNPhi + e] = -dt * fma(jb, K2, fma(-eb, K, id));
+      n[kNV + e] = 0.0;
+      n[kNP + e] = 0.0;
+      n[kNVa + e] = diag ? -dt : 0.0;
+      n[kNPa + e] = diag ? -hdt * dt : 0.0;
+      if (e == 0) n[kNT] = dt;
+    }
   bar_sync<1, 128>();
 }
 
@@ -158,58 +193,105 @@ __device__ void fast_leaves(FastSmem& S, int np, const double* bg, const double*
 //   Va = Va1 + R1 Va2, Pa = Pa1 + Va1 T2 + R1 Pa2, T = T1 + T2
 // over a binary tree of the np leaves: ceil(log2 np) levels of 6 dependent FP64
 // instructions each, one output element per lane (the prefix scans and sums of
-// the sequential order take 14 dependent ones per sum besides the scans).
-// Warps 0-3; returns the root.
+// the sequential order take 14 dependent ones per sum besides the scans).  64
+// lanes take a pair's 61 elements, two pairs per pass; a lane's element is the
+// same in every pass, so where its operands lie in the pair is worked out once
+// (worked out per element it took three times the FP64 arithmetic: 11.9k cycles
+// for 14 pieces).  Warps 0-3; returns the root.
 __device__ const double* fast_tree(FastSmem& S, int np) {
   const int t = threadIdx.x;
+  // first half: element xe of the pair's 18 X, pair t / 18 of 7 per pass
+  const int x0 = t / 18, xe = t - 18 * x0;
+  int xv1, xv2, xp1, xp2, xb;
+  {
+    const bool pos = xe >= 9;
+    const int q = pos ? xe - 9 : xe, r = q / 3, c = q - 3 * r;
+    const int r1 = r == 2 ? 0 : r + 1, r2 = r == 0 ? 2 : r - 1;
+    const int v = kNode + (pos ? kNp : kNv);                  // of the second run
+    xv1 = v + r1;
+    xv2 = v + r2;
+    xp1 = kNPhi + 3 * r1 + c;
+    xp2 = kNPhi + 3 * r2 + c;
+    xb = kNode + (pos ? kNP : kNV) + q;
+  }
+  // second half: element e of the pair, pair t / 64 of 2 per pass; operands as
+  // offsets from the first run's node (the second's follows it): three products
+  // A B along strides sa, sb, the base and the factor of T2 (kZero: none)
+  const int e = t & 63;
+  int oa, sa, ob, sb, obase, oext;
+  bool inX = false;
+  constexpr int kZero = -1;
+  {
+    const bool vec = e >= kNv;
+    const int f = vec ? (e - kNv) / 3 : e / 9;                // field
+    const int q = vec ? (e - kNv) - 3 * f : e - 9 * f;
+    const int r = vec ? q : q / 3, c = vec ? 0 : q - 3 * r;
+    const bool phi = !vec && f == 1;
+    oa = phi ? kNode + r : 3 * r;                             // row r of R1, or of R2^T
+    sa = phi ? 3 : 1;
+    sb = vec ? 1 : 3;
+    obase = (!vec && f == 0) ? kZero : phi ? kNode + e : e;
+    oext = kZero;
+    if (vec) {
+      ob = kNode + (f == 0 ? kNv : kNp);
+      if (f == 1) oext = kNv + q;
+    } else if (f == 0) {
+      ob = kNode + kNR + c;
+    } else if (phi) {
+      ob = kNPhi + c;
+    } else if (f == 2 || f == 3) {
+      inX = true;
+      ob = (f == 2 ? 0 : 9) + c;
+      if (f == 3) oext = kNV + q;
+    } else {
+      ob = kNode + (f == 4 ? kNVa : kNPa) + c;
+      if (f == 5) oext = kNVa + q;
+    }
+    if (e >= kNT) {                  // T (and the spare lanes): no products
+      oa = ob = sa = sb = 0;
+      oext = obase = kZero;
+      inX = false;
+    }
+  }
   double(*in)[kNode] = S.nodeA;
   double(*out)[kNode] = S.nodeB;
   for (int n = np; n > 1; n = (n + 1) >> 1) {
     const int full = n >> 1;
-    for (int L = t; L < 18 * full; L += 128) {
-      const int i = L / 18, e = L - 18 * i;
-      const double* n1 = in[2 * i];
-      const double* n2 = in[2 * i + 1];
-      const bool pos = e >= 9;
-      const int q = pos ? e - 9 : e, r = q / 3, c = q - 3 * r;
-      const int r1 = r == 2 ? 0 : r + 1, r2 = r == 0 ? 2 : r - 1;
-      const double* v = n2 + (pos ? kNp : kNv);
-      // minus row r of [v]x Phi1: -(v_r1 Phi_r2 - v_r2 Phi_r1)
-      S.X[i][e] = fma(v[r2], n1[kNPhi + 3 * r1 + c],
-                      fma(-v[r1], n1[kNPhi + 3 * r2 + c], n2[(pos ? kNP : kNV) + q]));
-    }
-    bar_sync<1, 128>();
-    for (int L = t; L < kNode * full; L += 128) {
-      const int i = L / kNode, e = L - kNode * i;
-      const double* n1 = in[2 * i];
-      const double* n2 = in[2 * i + 1];
-      double v;
-      if (e == kNT) {
-        v = n1[kNT] + n2[kNT];
-      } else {
-        const bool vec = e >= kNv;
-        const int f = vec ? (e - kNv) / 3 : e / 9;              // field
-        const int q = vec ? (e - kNv) - 3 * f : e - 9 * f;
-        const int r = vec ? q : q / 3, c = vec ? 0 : q - 3 * r;
-        const bool phi = !vec && f == 1;
-        const double* A = phi ? n2 + r : n1 + 3 * r;            // row r of R1, or of R2^T
-        const int sa = phi ? 3 : 1;
-        const double* B;
-        if (vec) B = n2 + (f == 0 ? kNv : kNp);
-        else if (f == 0) B = n2 + kNR + c;
-        else if (f == 1) B = n1 + kNPhi + c;
-        else if (f == 2 || f == 3) B = S.X[i] + (f == 2 ? 0 : 9) + c;
-        else B = n2 + (f == 4 ? kNVa : kNPa) + c;
-        const int sb = vec ? 1 : 3;
-        const double base = (!vec && f == 0) ? 0.0 : phi ? n2[e] : n1[e];
-        const bool lin = vec ? f == 1 : (f == 3 || f == 5);     // the T2-weighted velocity term
-        const double ve = lin ? n1[vec ? kNv + q : (f == 3 ? kNV : kNVa) + q] : 0.0;
-        v = fma(ve, n2[kNT], fma(A[0], B[0], fma(A[sa], B[sb], fma(A[2 * sa], B[2 * sb], base))));
+    if (x0 < 7)
+      for (int i = x0; i < full; i += 7) {
+        const double* b = in[2 * i];
+        // minus row r of [v2]x Phi1: -(v_r1 Phi_r2 - v_r2 Phi_r1)
+        S.X[i][xe] = fma(b[xv2], b[xp1], fma(-b[xv1], b[xp2], b[xb]));
       }
-      out[i][e] = v;
+    bar_sync<1, 128>();
+    for (int i = t >> 6; i < full; i += 4) {       // two pairs: the second's operands load beside the first's products
+      double a[2][3], bb[2][3], base[2], ext[2], T2[2], T1[2];
+      const bool two = i + 2 < full;
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int p = (u && two) ? i + 2 : i;
+        const double* b = in[2 * p];
+        const double* B = (inX ? S.X[p] : b) + ob;
+        const double* A = b + oa;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          a[u][k] = A[k * sa];
+          bb[u][k] = B[k * sb];
+        }
+        base[u] = obase < 0 ? 0.0 : b[obase];
+        ext[u] = oext < 0 ? 0.0 : b[oext];
+        T1[u] = b[kNT];
+        T2[u] = b[kNode + kNT];
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        if (u && !two) break;
+        const double v = e == kNT ? T1[u] + T2[u]
+                                  : fma(ext[u], T2[u], fma(a[u][0], bb[u][0], fma(a[u][1], bb[u][1], fma(a[u][2], bb[u][2], base[u]))));
+        if (e < kNode) out[i + 2 * u][e] = v;
+      }
     }
-    if (n & 1)                       // the odd run out moves up unchanged
-      for (int e = t; e < kNode; e += 128) out[full][e] = in[n - 1][e];
+    if ((n & 1) && t < kNode) out[full][t] = in[n - 1][t];    // the odd run out moves up unchanged
     bar_sync<1, 128>();
     double(*s)[kNode] = in;
     in = out;
@@ -309,9 +391,9 @@ __device__ __forceinline__ double fast_jlinv_e(const double* w0, double s, int e
   const double t2 = fma(w[0], w[0], fma(w[1], w[1], w[2] * w[2]));
   const int r = e / 3, q = e - 3 * r;
   double c;
-  if (t2 < 1e-5) {
+  if (pos_less(t2, 1e-5)) {
     c = fma(t2, fma(t2, 1.0 / 30240, 1.0 / 720), 1.0 / 12);
-  } else if (t2 < kSeriesT2) {
+  } else if (pos_less(t2, kSeriesT2)) {
     c = 1.0 / 12 + t2 * (1.0 / 720 + t2 * (1.0 / 30240 + t2 * (1.0 / 1209600 + t2 * (1.0 / 47900160))));
   } else {
     const double t = sqrt(t2);
@@ -331,19 +413,23 @@ __device__ void fast_state_terms(const SolveParams& sp, FastSmem& S) {
       quat_rot_e(g3 == 0 ? S.x0.q : g3 == 1 ? S.x0.qg : S.x1.q, e9);
   else if (lane < 30) S.c[lane - 27] = fma(S.x0.v[lane - 27], T, lane == 29 ? -0.5 * sp.g * T * T : 0.0);
   __syncwarp();
-  if (lane < 27) (g3 == 0 ? S.A0 : g3 == 1 ? S.QR : S.RcR1T)[e9] =
-      mm_e(g3 == 0 ? S.R0 : g3 == 1 ? S.Q0 : Rc, g3 == 0 ? Rc : g3 == 1 ? S.R0 : S.R1, e9, g3 == 2, g3 == 2);
-  else if (lane < 30) S.dr[lane - 27] = S.x1.r[lane - 27] - S.x0.r[lane - 27];
+  const int r3 = e9 / 3, c3 = e9 - 3 * r3;
+  if (lane < 27) {                   // A0 = R0 Rc, QR = Q0 R0, Rc^T R1^T
+    const double* A = g3 == 0 ? S.R0 + 3 * r3 : g3 == 1 ? S.Q0 + 3 * r3 : Rc + r3;
+    const double* B = g3 == 0 ? Rc + c3 : g3 == 1 ? S.R0 + c3 : S.R1 + 3 * c3;
+    (g3 == 0 ? S.A0 : g3 == 1 ? S.QR : S.RcR1T)[e9] = dot3(0.0, A, g3 == 2 ? 3 : 1, B, g3 == 2 ? 1 : 3);
+  } else if (lane < 30) {
+    S.dr[lane - 27] = S.x1.r[lane - 27] - S.x0.r[lane - 27];
+  }
   __syncwarp();
-  if (lane < 9) {
-    S.QA[lane] = mm_e(S.QR, Rc, lane, false, false);
-  } else if (lane < 18) {
-    const int k = (lane - 9) / 3, i = (lane - 9) % 3;
-    const double* A = k == 0 ? S.R0 : k == 1 ? S.Q0 : Rc;
-    const double* x = k == 1 ? S.c : sp.r_CS;
-    (k == 0 ? S.t1 : k == 1 ? S.t2c : S.rcS)[i] = mv_e(A, x, i, k != 0);
+  if (lane < 18) {                   // QA = QR Rc, t1 = R0 rc, t2 = Q0^T c, Rc^T rc
+    const int k = lane < 9 ? 0 : 1 + (lane - 9) / 3, i = (lane - 9) % 3;
+    const double* A = k == 0 ? S.QR + 3 * r3 : k == 1 ? S.R0 + 3 * i : k == 2 ? S.Q0 + i : Rc + i;
+    const double* B = k == 0 ? Rc + c3 : k == 2 ? S.c : sp.r_CS;
+    double* out = k == 0 ? S.QA + e9 : k == 1 ? S.t1 + i : k == 2 ? S.t2c + i : S.rcS + i;
+    *out = dot3(0.0, A, k < 2 ? 1 : 3, B, k == 0 ? 3 : 1);
   } else if (lane < 27) {
-    S.Jyr[e9 / 3][e9 % 3] = T * S.Q0[3 * (e9 % 3) + e9 / 3];          // position by velocity: T Q0^T
+    S.Jyr[r3][c3] = T * S.Q0[3 * c3 + r3];                    // position by velocity: T Q0^T
   }
   __syncwarp();
   double hr = 0.0;
@@ -358,6 +444,9 @@ __device__ void fast_state_terms(const SolveParams& sp, FastSmem& S) {
   } else if (lane < 27) {
     const int i = lane - 21;
     S.eb[i] = i < 3 ? S.x0.bg[i] - S.x1.bg[i] : S.x0.ba[i - 3] - S.x1.ba[i - 3];
+  } else if (lane < 30) {
+    const int i = lane - 27;         // velocity error without its pre-integrated part
+    S.evb[i] = fma(i == 2 ? -sp.g : 0.0, T, S.x0.v[i]) - S.x1.v[i];
   }
   // C: the photometric local Jacobian on p0, -[R0 0; [dr]x R0, R0], and on p1,
   // diag(R0, R0); the ICP one on p1, diag(R_ref, R_ref)
@@ -411,7 +500,7 @@ __device__ void fast_gravity(FastSmem& S, bool gyro) {
     for (int k = 0; k < 3; ++k) v = fma(S.nv[k], lane < 2 ? S.Jlg[3 * k + lane] : S.eg[k], v);
     v = gyro ? 0.0 : v * inv;
     if (lane < 2) S.a[lane] = v;
-    else S.s = v;
+    else S.s = v, S.a[2] = 0.0;
   } else if (lane < 9) {             // Gm row m, column k; det(B^T B) = |n|^2 (Lagrange's identity)
     const int m = (lane - 3) / 3, k = (lane - 3) % 3;
     const double det = fma(S.mm[0], S.mm[2], -(S.mm[1] * S.mm[1]));
@@ -486,30 +575,157 @@ __device__ void fast_pixel_terms(const SolveParams& sp, const Ctrl* c, FastSmem&
 
 // ---- the sweep ---------------------------------------------------------------------
 
-// 1 / |d| as pivot_recip, sign restored.
-__device__ __forceinline__ double signed_recip(double d, bool neg) {
-  const double r = pivot_recip(neg ? -d : d);
-  return neg ? -r : r;
+// x <- x boxplus d by one warp, as warp_state_boxplus: the series of a quaternion
+// group's four components run on its four lanes (cosine on the first, sine on the
+// others), cut where the next term is below 1e-17 for small steps.
+__device__ __forceinline__ void fast_boxplus(DState& x, const double* d) {
+  const int lane = threadIdx.x & 31, grp = (lane >> 2) & 1, k = lane & 3, base = lane & ~3;
+  double* q = grp ? x.qg : x.q;
+  const double d0 = grp ? d[15] : d[3], d1 = grp ? d[16] : d[4], d2 = grp ? 0.0 : d[5];
+  const double t2 = fma(d0, d0, fma(d1, d1, d2 * d2));
+  double f;
+  if (__all_sync(0xffffffffu, pos_less(t2, 1e-6))) {
+    f = fma(t2, fma(t2, k ? 1.0 / 3840 : 1.0 / 384, k ? -1.0 / 48 : -1.0 / 8), k ? 0.5 : 1.0);
+  } else if (__all_sync(0xffffffffu, pos_less(t2, kSeriesT2))) {
+    const double c4 = k ? 1.0 / 185794560 : 1.0 / 10321920, c3 = k ? -1.0 / 645120 : -1.0 / 46080;
+    const double c2 = k ? 1.0 / 3840 : 1.0 / 384, c1 = k ? -1.0 / 48 : -1.0 / 8;
+    f = fma(t2, fma(t2, fma(t2, fma(t2, c4, c3), c2), c1), k ? 0.5 : 1.0);
+  } else {
+    const double t = sqrt(t2);
+    double sn, cs;
+    sincos(0.5 * t, &sn, &cs);
+    f = k ? (t2 > 0.0 ? sn / t : 0.5) : cs;
+  }
+  f *= k == 0 ? 1.0 : k == 1 ? d0 : k == 2 ? d1 : d2;
+  double o = 0.0;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {      // component k of exp(d) (x) q, as quat_mul_k
+    const double e = __shfl_sync(0xffffffffu, f, base + j);
+    o = fma(((0x428E >> (4 * k + j)) & 1) ? -e : e, q[k ^ j], o);
+  }
+  double n2 = o * o;
+  n2 += __shfl_xor_sync(0xffffffffu, n2, 1);
+  n2 += __shfl_xor_sync(0xffffffffu, n2, 2);
+  if (__all_sync(0xffffffffu, fabs(__double2float_rn(n2) - 1.f) < 1e-6f)) o *= fma(-0.5, n2, 1.5);
+  else o *= rsqrt(n2);
+  __syncwarp();
+  if (lane < 8) q[k] = o;
+  if (lane < 12) {
+    const int g = lane / 3, i = lane - 3 * g;
+    double* v = g == 0 ? x.r : g == 1 ? x.v : g == 2 ? x.bg : x.ba;
+    v[i] += d[(g == 0 ? 0 : 3 + 3 * g) + i];
+  }
+  __syncwarp();
 }
 
-// One Gauss-Newton step (every thread of the block); status and all that is
-// uniform has been checked by the caller.
-__device__ void gn_step_fast(const SolveParams& sp, Ctrl* c, FastSmem& S) {
+// The pixel kernel's transforms, as warp_write_transforms, from shared memory; warp 0.
+__device__ __forceinline__ void fast_transforms(Ctrl* c, FastSmem& S) {
+  const int lane = threadIdx.x & 31, f = lane / 9, e = lane - 9 * f, r = e / 3, cc = e - 3 * r;
+  if (lane < 24) {                    // R1, R0 (2 (v_r v_c + w^2 or +- w v_k) - I); r1 - r_ref, r1 - r0
+    const double* q = f == 0 ? S.x1.q : S.x0.q;
+    const bool rot = lane < 18, diag = r == cc, icp = lane < 21;
+    const int i = (lane - 18) % 3;
+    const double w = q[0], vk = diag ? w : q[4 - r - cc];
+    const double x = rot ? w * ((((cc - r + 3) % 3) == 1) ? -vk : vk) : icp ? -S.rref[i] : -S.x0.r[i];
+    const double h = fma(rot ? q[1 + r] : S.x1.r[i], rot ? q[1 + cc] : 1.0, x);
+    S.rot[lane] = rot ? fma(2.0, h, diag ? -1.0 : 0.0) : h;
+  }
+  __syncwarp();
+  const double* R1 = S.rot;
+  const double* R0 = S.rot + 9;
+  if (lane < 24) {
+    const bool rot = lane < 18, icp = rot ? f == 0 : lane < 21;
+    const int i = rot ? r : (lane - 18) % 3;
+    const double* M = (icp ? S.Rref : R0) + i;                // column i: row i of the transpose
+    const double* B = rot ? R1 + cc : S.rot + (icp ? 18 : 21);
+    const double v = dot3(rot && r == cc ? -1.0 : 0.0, M, 3, B, rot ? 3 : 1);
+    (icp ? c->xf_icp : c->xf_rgb)[rot ? e : 9 + i] = (float)v;
+  }
+}
+
+// One Gauss-Newton step; false (for every thread, nothing done) when the frame's
+// constants do not allow this form.  Whole block.
+__device__ bool gn_step_fast(const SolveParams& sp, FastSmem& S) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const bool gyro = sp.track_mode == DRI_TRACK_GYRO_ONLY;
-  {                                   // one round of independent loads
+  Ctrl* c = sp.ctrl;
+  const int status = c->status, usable = c->elim.ok, np = c->elim.np;
+  {                                   // everything in one round of independent loads
     const double* e = c->elim.m;
-    for (int i = tid; i < kElimDoubles; i += kSolveThreads) S.el[i] = e[i];
     const double* p = &c->elim.piece[0][0];
     double* q = &S.piece[0][0];
-#pragma unroll
-    for (int i = 0; i < kElimPieces * 8 / kSolveThreads; ++i) q[tid + i * kSolveThreads] = p[tid + i * kSolveThreads];
-    if (tid < 20) reinterpret_cast<double*>(&S.x0)[tid] = reinterpret_cast<const double*>(&c->x0)[tid];
-    else if (tid < 40) reinterpret_cast<double*>(&S.x1)[tid - 20] = reinterpret_cast<const double*>(&c->x1)[tid - 20];
-    else if (tid < 60) reinterpret_cast<double*>(&S.xbar)[tid - 40] = reinterpret_cast<const double*>(&c->xbar)[tid - 40];
-    else if (tid >= 64 && tid < 73) S.Rref[tid - 64] = c->Rref[tid - 64];
+    double v[4];
+    v[0] = p[tid];
+    v[1] = p[tid + kSolveThreads];
+    v[2] = e[tid];
+    v[3] = 0.0;
+    static_assert(kElimPieces * 8 == 2 * kSolveThreads && kElimDoubles - kSolveThreads == 40, "load layout");
+    const double* src = tid < 20 ? reinterpret_cast<const double*>(&c->x0) + tid
+                        : tid < 40 ? reinterpret_cast<const double*>(&c->x1) + tid - 20
+                        : tid < 60 ? reinterpret_cast<const double*>(&c->xbar) + tid - 40
+                        : tid < 69 ? c->Rref + tid - 60
+                        : tid < 109 ? e + kSolveThreads + tid - 69
+                        : tid < 112 ? c->rref + tid - 109 : nullptr;
+    double* dst = tid < 20 ? reinterpret_cast<double*>(&S.x0) + tid
+                  : tid < 40 ? reinterpret_cast<double*>(&S.x1) + tid - 20
+                  : tid < 60 ? reinterpret_cast<double*>(&S.xbar) + tid - 40
+                  : tid < 69 ? S.Rref + tid - 60
+                  : tid < 109 ? S.el + kSolveThreads + tid - 69 : S.rref + tid - 109;
+    if (src) v[3] = *src;
+    q[tid] = v[0];
+    q[tid + kSolveThreads] = v[1];
+    S.el[tid] = v[2];
+    if (src) *dst = v[3];
   }
-  const int np = c->elim.np;
+  if (status != 0) return true;
+  if (!usable) {
+    __syncthreads();                  // the other form reuses this shared memory
+    return false;
+  }
+  // the sweep's entries of this thread (see there): entry e of the lower triangle
+  // and the right-hand side row, longest-updated first, and where its value comes
+  // from: sign (*p + *q)
+  int ei[2], ej[2];
+  const double *ep[2], *eq[2];
+  bool eneg[2];
+#pragma unroll
+  for (int o = 0; o < 2; ++o) {
+    const int e = tid + 128 * o;
+    ei[o] = ej[o] = -1;
+    ep[o] = eq[o] = &S.zero;
+    eneg[o] = false;
+    if (warp < 4 && e < kSysEnt) {    // column j = 18 - g holds rows j .. 19 (19: right-hand side): g + 2 entries
+      int g = (int)((sqrtf(9.0f + 8.0f * e) - 3.0f) * 0.5f);
+      if (g * (g + 3) / 2 > e) --g;
+      if ((g + 1) * (g + 4) / 2 <= e) ++g;
+      ej[o] = kSys - 1 - g;
+      ei[o] = ej[o] + e - g * (g + 3) / 2;
+      const int i = ei[o], j = ej[o];
+      if (i < kLam) {                 // -(S + blockdiag(S6, sigma_g^2))
+        ep[o] = S.S + tri(i, j);
+        eneg[o] = true;
+        if (i < 6) eq[o] = S.el + kElS6 + 6 * i + j;
+        else if (i == j) eq[o] = S.el + kElSg;
+      } else if (j < kLam) {          // J', -e'
+        ep[o] = i == kSys ? S.ep + j : &S.Jp[j][i - kLam];
+        eneg[o] = i == kSys;
+      } else if (i == kSys) {         // the prior on p0
+        if (j < kLam + 6) ep[o] = S.bp + j - kLam;
+      } else if (i < kLam + 6) {
+        ep[o] = S.el + kElHp + 6 * (i - kLam) + j - kLam;
+      }
+    }
+  }
+  if (tid == 0) {
+    S.one = 1.0;
+    S.zero = 0.0;
+  }
+  // J' on p1: -I for the position rows, zero where the rotation rows do not write
+  if (warp == 4)
+    for (int idx = lane; idx < 42; idx += 32) {
+      const int i = idx / 6, k = idx - 6 * i;
+      if (i < 3 || i == 6 || k < 3) S.Jp[i][6 + k] = (i < 3 && k == i && !gyro) ? -1.0 : 0.0;
+    }
   __syncthreads();
   const double* root = nullptr;
   if (warp < 4) {
@@ -554,30 +770,29 @@ __device__ void gn_step_fast(const SolveParams& sp, Ctrl* c, FastSmem& S) {
   } else {
     // ---- IMU rows ----
     if (warp == 0) {
-      const int g3 = lane / 9, e9 = lane - 9 * g3;
-      if (lane < 9) {
-        S.RW[lane] = mm_e(S.A0, root + kNR, lane, false, false);
-      } else if (lane < 18) {         // position by b_a
-        S.Jyr[e9 / 3][6 + e9 % 3] = mm_e(S.A0, root + kNPa, e9, false, false);
-      } else if (lane < 27) {
-        S.APg[e9] = mm_e(S.A0, root + kNP, e9, false, false);
-      } else if (lane < 30) {
-        S.t3[lane - 27] = mv_e(S.A0, root + kNp, lane - 27, false);
+      const int f = lane / 9, e9 = lane - 9 * f, r = f == 3 ? e9 : e9 / 3, cc = f == 3 ? 0 : e9 - 3 * r;
+      if (lane < 30) {                // A0 times R, Pa (position by b_a), P, p
+        const double* B = root + (f == 0 ? kNR : f == 1 ? kNPa : f == 2 ? kNP : kNp) + cc;
+        double* out = f == 0 ? S.RW + e9 : f == 1 ? &S.Jyr[r][6 + cc] : f == 2 ? S.APg + e9 : S.t3 + e9;
+        *out = dot3(0.0, S.A0 + 3 * r, 1, B, f == 3 ? 1 : 3);
       }
       __syncwarp();
-      if (lane < 9) S.M[lane] = mm_e(S.RW, S.RcR1T, lane, false, false);
-      else if (lane < 18) S.RP[e9] = mm_e(S.RW, root + kNPhi, e9, false, false);
-      else if (lane < 21) S.t4[lane - 18] = mv_e(S.RW, S.rcS, lane - 18, false);
+      if (lane < 21) {                // R_WS1 times Rc^T R1^T, Phi, Rc^T rc
+        const int rr = f == 2 ? e9 : r;
+        const double* B = f == 0 ? S.RcR1T + cc : f == 1 ? root + kNPhi + cc : S.rcS;
+        double* out = f == 0 ? S.M + e9 : f == 1 ? S.RP + e9 : S.t4 + e9;
+        *out = dot3(0.0, S.RW + 3 * rr, 1, B, f == 2 ? 1 : 3);
+      }
       __syncwarp();
-      if (lane < 9) {                 // position by b_g
-        const double v = S.APg[lane] + hatm_e(S.t4, S.RP, lane);
-        S.Jyr[lane / 3][3 + lane % 3] = v;
-      } else if (lane < 12) {
-        const int i = lane - 9;
-        S.er[i] = (S.base[i] + S.t3[i]) - S.t4[i];
-      } else if (lane < 15) {
-        const int i = lane - 12;
-        S.u[i] = (S.t1[i] + S.t3[i]) - S.t4[i];
+      if (lane < 15) {                // position by b_g: A0 P + [t4]x R_WS1 Phi; e_r; u = t1 + t3 - t4
+        const int i = lane < 12 ? lane - 9 : lane - 12;
+        const int r1 = r == 2 ? 0 : r + 1, r2 = r == 0 ? 2 : r - 1;
+        const bool mat = lane < 9;
+        const double x = mat ? S.APg[lane] : lane < 12 ? S.base[i] : S.t1[i];
+        const double y1 = mat ? S.t4[r1] : 1.0, z1 = mat ? S.RP[3 * r2 + cc] : S.t3[i];
+        const double y2 = mat ? S.t4[r2] : 1.0, z2 = mat ? S.RP[3 * r1 + cc] : S.t4[i];
+        double* out = mat ? &S.Jyr[r][3 + cc] : lane < 12 ? S.er + i : S.u + i;
+        *out = fma(-y2, z2, fma(y1, z1, x));
       }
       __syncwarp();
       if (gyro) {                     // the position rows carry no weight: no information
@@ -595,29 +810,37 @@ __device__ void gn_step_fast(const SolveParams& sp, Ctrl* c, FastSmem& S) {
                      v2 = __shfl_sync(0xffffffffu, v, 2);
         const double s2 = fma(v0, v0, fma(v1, v1, v2 * v2));
         const float tr = (float)S.M[0] + (float)S.M[4] + (float)S.M[8];
-        if (s2 < 4e-5 && tr > 2.f) ea = v * fma(s2, fma(s2, fma(s2, 5.0 / 112, 3.0 / 40), 1.0 / 6), 1.0);
+        if (pos_less(s2, 4e-5) && tr > 2.f) ea = v * fma(s2, fma(s2, fma(s2, 5.0 / 112, 3.0 / 40), 1.0 / 6), 1.0);
         else ea = log_i(S.M, i);
       }
       if (lane < 3) S.ea[lane] = ea;
       __syncwarp();
-      if (lane < 18) (lane < 9 ? S.Jla : S.Jra)[e9] = fast_jlinv_e(S.ea, lane < 9 ? 1.0 : -1.0, e9);
-      __syncwarp();
-      if (lane < 9) S.B13[lane] = mm_e(S.Jla, S.RP, lane, false, false);
-    } else if (warp == 3) {           // velocity rows, used for dv1 only
-      if (lane < 9) S.B14[lane] = mm_e(S.QA, root + kNV, lane, false, false);
-      else if (lane < 18) S.B17[lane - 9] = mm_e(S.QA, root + kNVa, lane - 9, false, false);
-      else if (lane < 24) {
-        const int k = (lane - 18) / 3, i = (lane - 18) % 3;
-        (k == 0 ? S.w9 : S.t5)[i] = mv_e(k == 0 ? S.A0 : S.QA, root + kNv, i, false);
+      if (lane < 18) {                // Jl^-1(e_a), and -Jr^-1(e_a) into J' on p1
+        const double v = fast_jlinv_e(S.ea, lane < 9 ? 1.0 : -1.0, e9);
+        if (lane < 9) S.Jla[e9] = v;
+        else S.Jp[3 + r][9 + cc] = -v;
       }
       __syncwarp();
-      if (lane < 9) S.B9[lane] = -mhat_e(S.Q0, false, S.w9, lane);
-      else if (lane < 18) {
-        const int e = lane - 9;
-        if (e % 3 < 2) S.B20[2 * (e / 3) + e % 3] = -hat_e(S.t5, e);
+      if (lane < 9) S.B13[lane] = dot3(0.0, S.Jla + 3 * r, 1, S.RP + cc, 3);
+    } else if (warp == 3) {           // velocity rows, used for dv1 only
+      const int f = lane / 9, e9 = lane - 9 * f, r = f < 2 ? e9 / 3 : e9 % 3, cc = f < 2 ? e9 - 3 * r : 0;
+      if (lane < 24) {                // QA V, QA Va, A0 v, QA v
+        const double* A = (f == 2 && e9 < 3 ? S.A0 : S.QA) + 3 * r;
+        const double* B = root + (f == 0 ? kNV : f == 1 ? kNVa : kNv) + cc;
+        double* out = f == 0 ? S.B14 + e9 : f == 1 ? S.B17 + e9 : e9 < 3 ? S.w9 + r : S.t5 + r;
+        *out = dot3(0.0, A, 1, B, f == 2 ? 1 : 3);
+      }
+      __syncwarp();
+      if (lane < 12) {                // -Q0 [w9]x, e_v
+        const int c1 = cc == 2 ? 0 : cc + 1, c2 = cc == 0 ? 2 : cc - 1, i = lane - 9;
+        const bool mat = lane < 9;
+        const double x = mat ? 0.0 : S.evb[i];
+        const double y1 = mat ? S.Q0[3 * r + c1] : 0.0, z1 = mat ? S.w9[c2] : 0.0;
+        const double y2 = mat ? S.Q0[3 * r + c2] : 1.0, z2 = mat ? S.w9[c1] : S.t5[i];
+        *(mat ? S.B9 + lane : S.ev + i) = fma(y2, z2, fma(-y1, z1, x));
       } else if (lane < 21) {
-        const int i = lane - 18;
-        S.ev[i] = (fma(i == 2 ? -sp.g : 0.0, S.el[kElT], S.x0.v[i]) + S.t5[i]) - S.x1.v[i];
+        const int q = lane - 12;
+        if (q % 3 < 2) S.B20[2 * (q / 3) + q % 3] = -hat_e(S.t5, q);
       }
     }
     if (warp == 1 || warp == 2) {     // position rows: Jy P, Jp + Jy K, e + Jy m
@@ -650,24 +873,34 @@ __device__ void gn_step_fast(const SolveParams& sp, Ctrl* c, FastSmem& S) {
       bar_sync<5, 96>();
       // rotation rows (their only y column block is b_g: B13) and the gravity row
       if (warp == 0) {
-        if (lane < 9) {
-          const int i = lane / 3, j = lane - 3 * i;
-          double v = 0.0;
-#pragma unroll
-          for (int k = 0; k < 3; ++k) v = fma(S.B13[3 * i + k], S.T[j][3 + k], v);
-          S.S[tri(3 + i, j)] = v;
+        const int i = lane / 3, j = lane - 3 * i;
+        const bool rot = lane < 9;    // S between the rotation and position rows; else the gravity row
+        const double* A = rot ? S.B13 + 3 * i : S.a;
+        const double* B;
+        double* out;
+        int sb = 1;
+        double base = 0.0;
+        if (rot) {
+          B = &S.T[j][3];
+          out = S.S + tri(3 + i, j);
         } else if (lane < 20) {
-          const int q = lane - 9;
-          S.T[6][q] = fma(S.a[0], Py[9 * 11 + q], S.a[1] * Py[10 * 11 + q]);
+          B = Py + 9 * 11 + lane - 9;
+          sb = 11;
+          out = &S.T[6][lane - 9];
         } else if (lane < 23) {
-          const int j = lane - 20;
-          S.S[tri(6, j)] = fma(S.a[0], S.T[j][9], S.a[1] * S.T[j][10]);
+          B = &S.T[lane - 20][9];
+          out = S.S + tri(6, lane - 20);
         } else if (lane < 29) {
-          const int q = lane - 23;
-          S.Jp[6][q] = fma(S.a[0], K[9 * 6 + q], S.a[1] * K[10 * 6 + q]);
-        } else if (lane == 29) {
-          S.ep[6] = S.s + fma(S.a[0], S.m[9], S.a[1] * S.m[10]);
+          B = K + 9 * 6 + lane - 23;
+          sb = 6;
+          out = &S.Jp[6][lane - 23];
+        } else {
+          B = S.m + 9;
+          out = S.ep + 6;
+          base = S.s;
         }
+        const double v = dot21(base, A, B, sb, rot ? A + 2 : &S.zero, rot ? B + 2 : &S.zero);
+        if (lane < 30) *out = v;
       } else {
         const int q = lane - 11;
         const int r = warp == 1 ? lane / 11 : lane < 11 ? 2 : lane < 29 ? q / 6 : lane - 29;
@@ -685,104 +918,89 @@ __device__ void gn_step_fast(const SolveParams& sp, Ctrl* c, FastSmem& S) {
           else S.ep[3 + r] = v;
         }
       }
-      // the rows' constant parts on p1: -I, -Jr^-1
-      if (warp == 0)
-        for (int idx = lane; idx < 42; idx += 32) {
-          const int i = idx / 6, k = idx - 6 * i;
-          double v = 0.0;
-          if (i < 3) v = k == i && !gyro ? -1.0 : 0.0;
-          else if (i < 6 && k >= 3) v = -S.Jra[3 * (i - 3) + k - 3];
-          S.Jp[i][6 + k] = v;
-        }
       bar_sync<5, 96>();
-      if (warp == 1) {
-        if (lane < 6) {
-          const int i = lane < 1 ? 0 : lane < 3 ? 1 : 2, j = lane - tri(i, 0);
-          double v = 0.0;
-#pragma unroll
-          for (int k = 0; k < 3; ++k) v = fma(S.T[3 + i][3 + k], S.B13[3 * j + k], v);
-          S.S[tri(3 + i, 3 + j)] = v;
-        } else if (lane < 10) {       // gravity row against the rotation rows and itself
-          const int j = lane - 3;     // 3, 4, 5, 6
-          S.S[tri(6, j)] = fma(S.a[0], S.T[j][9], S.a[1] * S.T[j][10]);
-        }
+      if (warp == 1 && lane < 10) {   // S of the rotation rows; the gravity row against them and itself
+        const bool rot = lane < 6;
+        const int i = lane < 1 ? 0 : lane < 3 ? 1 : 2, j = rot ? lane - tri(i, 0) : lane - 3;
+        const double* A = rot ? &S.T[3 + i][3] : S.a;
+        const double* B = rot ? S.B13 + 3 * j : &S.T[j][9];
+        const double v = dot21(0.0, A, B, 1, rot ? A + 2 : &S.zero, rot ? B + 2 : &S.zero);
+        S.S[rot ? tri(3 + i, 3 + j) : tri(6, j)] = v;
       }
     }
     bar_arrive<7, 160>();
     bar_sync<1, 128>();
-    // ---- the sweep: entry e of the lower triangle and the right-hand side row,
-    // longest-updated first, 32-entry chunks dealt to the four warps in turn, so
-    // that the entries a pivot still updates take the fewest warp instructions ----
-    int ei[2], ej[2];
-    double v[2];
+    // ---- the sweep: the entries are dealt to the four warps in 32-entry chunks in
+    // turn, longest-updated first, so that the entries a pivot still updates take
+    // the fewest warp instructions: the second slot's 81 entries have columns 0..4
+    // and are done after pivot 3 ----
+    double v[2], rown[2] = {0.0, 0.0};
 #pragma unroll
     for (int o = 0; o < 2; ++o) {
-      const int e = tid + 128 * o;
-      int i = -1, j = -1;
-      double x = 0.0;
-      if (e < kSysEnt) {              // column j = 18 - g holds rows j .. 19 (19: right-hand side): g + 2 entries
-        int g = (int)((sqrtf(9.0f + 8.0f * e) - 3.0f) * 0.5f);
-        while (g * (g + 3) / 2 > e) --g;
-        while ((g + 1) * (g + 4) / 2 <= e) ++g;
-        j = kSys - 1 - g;
-        i = j + e - g * (g + 3) / 2;
-        if (i < kLam) {               // -(S + blockdiag(S6, sigma_g^2))
-          const double s6 = i < 6 ? S.el[kElS6 + 6 * i + j] : i == j ? S.el[kElSg] : 0.0;
-          x = -(S.S[tri(i, j)] + s6);
-        } else if (j < kLam) {
-          x = i == kSys ? -S.ep[j] : S.Jp[j][i - kLam];
-        } else if (i == kSys) {
-          x = j < kLam + 6 ? S.bp[j - kLam] : 0.0;
-        } else {
-          x = i < kLam + 6 ? S.el[kElHp + 6 * (i - kLam) + j - kLam] : 0.0;
-        }
-      }
-      ei[o] = i;
-      ej[o] = j;
-      v[o] = x;
+      const double x = *ep[o] + *eq[o];
+      v[o] = eneg[o] ? -x : x;
     }
-    for (int k = 0; k < kSys; ++k) {
-      if (k == kLam) {                // the pixel terms join the pose block
-        grid_dep_wait();
-        bar_sync<4, 256>();
-#pragma unroll
-        for (int o = 0; o < 2; ++o) {
-          const int i = ei[o], j = ej[o];
-          if (j >= kLam) v[o] += i == kSys ? S.g12[j - kLam] : S.P12[(i - kLam) * kPose + j - kLam];
-        }
-      }
+    // Pivot k (slots 0 .. O - 1): its column is published behind one barrier; the
+    // products c_i c_j are taken while the reciprocal's seed is formed on the integer
+    // and FP32 pipes.  No branches: a lane without a column entry writes to its sink
+    // word, one whose entry is done keeps its value.
+    auto pivot = [&](int k, bool neg, auto slots) {
+      constexpr int O = decltype(slots)::value;
       double* cb = S.col[k & 1];
 #pragma unroll
-      for (int o = 0; o < 2; ++o)
-        if (ej[o] == k) cb[ei[o]] = v[o];
+      for (int o = 0; o < O; ++o) *(ej[o] == k ? cb + ei[o] : S.sink + tid) = v[o];
       bar_sync<1, 128>();
       const double d = cb[k];
-      const double r = signed_recip(d, k < kLam);
-      if (tid == 0) {
-        S.piv[k] = k < kLam ? -d : d;
-        S.rinv[k] = r;
+      double t[O];
+#pragma unroll
+      for (int o = 0; o < O; ++o) t[o] = cb[max(ei[o], 0)] * cb[max(ej[o], 0)];
+      const double r = pivot_recip(neg ? -d : d);             // 1 / |d|
+#pragma unroll
+      for (int o = 0; o < O; ++o) {
+        const double w = fma(neg ? t[o] : -t[o], r, v[o]);
+        v[o] = ej[o] > k ? w : v[o];
+        rown[o] = ej[o] == k ? (neg ? -r : r) : rown[o];
       }
-#pragma unroll
-      for (int o = 0; o < 2; ++o)
-        if (ej[o] > k) v[o] = fma(-(cb[ei[o]] * r), cb[ej[o]], v[o]);
+    };
+#pragma unroll 1
+    for (int k = 0; k < 5; ++k) pivot(k, true, Slots<2>());
+#pragma unroll 1
+    for (int k = 5; k < kLam; ++k) pivot(k, true, Slots<1>());
+    grid_dep_wait();
+    bar_sync<4, 256>();               // the pixel terms join the pose block (slot 0's columns)
+    {
+      const int i = ei[0], j = ej[0];
+      if (j >= kLam) v[0] += i == kSys ? S.g12[j - kLam] : S.P12[(i - kLam) * kPose + j - kLam];
     }
-    bar_sync<1, 128>();
+#pragma unroll 1
+    for (int k = kLam; k < kSys; ++k) pivot(k, false, Slots<1>());
+    // unit-lower L, its row 19 holding z_k / d_k; the pivots' signs
+    bool posdef = true;
 #pragma unroll
-    for (int o = 0; o < 2; ++o)       // unit-lower L; its row 19 holds z_k / d_k
-      if (ei[o] > ej[o]) S.L[ej[o]][ei[o]] = v[o] * S.rinv[ej[o]];
+    for (int o = 0; o < 2; ++o) {
+      if (ei[o] > ej[o]) S.L[ej[o]][ei[o]] = v[o] * rown[o];
+      if (ei[o] >= 0 && ei[o] == ej[o]) {
+        const bool neg = __double2hiint(v[o]) < 0;
+        posdef = posdef && finite_bits(v[o]) && v[o] != 0.0 && neg == (ei[o] < kLam);
+      }
+    }
+    posdef = __all_sync(0xffffffffu, posdef);
+    if (lane == 0) S.posdef[warp] = posdef;
     bar_sync<1, 128>();
     if (warp < 2) {
       double* dx = S.dx;
       if (warp == 0) {
-        double y = lane < kSys ? S.L[lane][kSys] : 0.0;
-        for (int k = kSys - 1; k > 0; --k) {
-          const double xk = __shfl_sync(0xffffffffu, y, k);
-          if (lane < k) y = fma(-S.L[lane][k], xk, y);
+        const double* Lr = S.L[min(lane, kSys - 1)];
+        double y = Lr[kSys], l = Lr[kSys - 1];
+#pragma unroll 1
+        for (int k = kSys - 1; k > 0; --k) {                  // the next column's entry loads a step ahead
+          const double ln = Lr[k - 1];
+          y = fma(lane < k ? -l : 0.0, __shfl_sync(0xffffffffu, y, k), y);
+          l = ln;
         }
         if (lane < kSys) S.z[lane] = y;
         if (lane >= kLam && lane < kSys) dx[lane < kLam + 6 ? lane - kLam : 4 + lane] = y;   // p0 at 0..5, p1 at 17..22
-        bool ok = lane >= kSys || (S.piv[lane] > 0.0 && S.piv[lane] < INFINITY);
-        ok = __all_sync(0xffffffffu, ok);
+        bool ok = S.posdef[0] && S.posdef[1] && S.posdef[2] && S.posdef[3];
         __syncwarp();
         // y (lanes 0-10: K p0 + m, 16-26: -T^T lambda), dv1's part without y
         // (11-13: e_v + B9 da0, 27-29: -S_v6 lambda)
@@ -806,31 +1024,40 @@ __device__ void gn_step_fast(const SolveParams& sp, Ctrl* c, FastSmem& S) {
         else if (lane < 14) S.u[lane - 11] = w;            // dv1's part
         __syncwarp();
         bool fin = true;
-        if (lane < 17) fin = ((__double_as_longlong(dx[lane]) >> 52) & 0x7ff) != 0x7ff;
+        if (lane < 17) fin = finite_bits(dx[lane]);
         ok = __all_sync(0xffffffffu, fin) && ok;
         if (lane == 0) S.good[0] = ok;
       }
       bar_sync<6, 64>();
       if (warp == 0) {
-        warp_state_boxplus(S.x0, dx);
+        fast_boxplus(S.x0, dx);
       } else {
         const double* y = dx + 6;     // v, b_g, b_a, gravity
-        double w = 0.0;
-        if (lane < 9) {               // dv1: row lane % 3, part lane / 3
-          const int i = lane % 3, q = lane / 3;
-          const double* A = q == 0 ? S.B14 + 3 * i : q == 1 ? S.B17 + 3 * i : S.B20 + 2 * i;
-          const double* B = q == 0 ? y + 3 : q == 1 ? y + 6 : y + 9;
-          w = q == 2 ? y[i] + S.u[i] : 0.0;
-#pragma unroll
-          for (int k = 0; k < 3; ++k)
-            if (k < 2 || q < 2) w = fma(A[k], B[k], w);
-        } else if (lane < 15) {       // x1's biases follow x0's
-          w = S.eb[lane - 9] + y[3 + lane - 9];
-          if (gyro && lane >= 12) w = 0.0;
+        // lanes 0-8: dv1, row lane % 3, part lane / 3; 9-14: x1's biases follow x0's;
+        // 15-17: e_g + A dg0
+        const int i = lane % 3, q = lane / 3;
+        const double *A = &S.zero, *B = &S.zero, *A2 = &S.zero, *B2 = &S.zero;
+        int sa = 0, sb = 0;
+        double base = 0.0;
+        if (lane < 9) {
+          A = q == 0 ? S.B14 + 3 * i : q == 1 ? S.B17 + 3 * i : S.B20 + 2 * i;
+          B = q == 0 ? y + 3 : q == 1 ? y + 6 : y + 9;
+          A2 = q == 2 ? &S.one : A + 2;
+          B2 = q == 2 ? y + i : B + 2;
+          base = q == 2 ? S.u[i] : 0.0;
+          sa = sb = 1;
+        } else if (lane < 15) {
+          A2 = &S.one;
+          B2 = y + 3 + lane - 9;
+          base = S.eb[lane - 9];
         } else if (lane < 18) {
-          const int i = lane - 15;
-          w = fma(S.Ag[2 * i], y[9], fma(S.Ag[2 * i + 1], y[10], S.eg[i]));
+          A = S.Ag + 2 * i;
+          B = y + 9;
+          base = S.eg[i];
+          sa = sb = 1;
         }
+        double w = fma(A[0], B[0], fma(A[sa], B[sb], fma(*A2, *B2, base)));
+        if (gyro && lane >= 12 && lane < 15) w = 0.0;
         const double w1 = __shfl_down_sync(0xffffffffu, w, 3), w2 = __shfl_down_sync(0xffffffffu, w, 6);
         const double u0 = __shfl_sync(0xffffffffu, w, 15), u1 = __shfl_sync(0xffffffffu, w, 16),
                      u2 = __shfl_sync(0xffffffffu, w, 17);
@@ -842,20 +1069,20 @@ __device__ void gn_step_fast(const SolveParams& sp, Ctrl* c, FastSmem& S) {
         }
         __syncwarp();
         bool fin = true;
-        if (lane < 17) fin = ((__double_as_longlong(dx[17 + lane]) >> 52) & 0x7ff) != 0x7ff;
+        if (lane < 17) fin = finite_bits(dx[17 + lane]);
         fin = __all_sync(0xffffffffu, fin);
         if (lane == 0) S.good[1] = fin;
-        warp_state_boxplus(S.x1, dx + 17);
+        fast_boxplus(S.x1, dx + 17);
       }
     }
   }
   __syncthreads();
   if (!S.good[0] || !S.good[1]) {
     if (tid == 0) c->status = DRI_ELOST;
-    return;
+    return true;
   }
   if (warp == 0) {
-    warp_write_transforms(c, S.x0, S.x1, S.rot);
+    fast_transforms(c, S);
   } else if (warp == 1) {
     if (lane < 20) reinterpret_cast<double*>(&c->x0)[lane] = reinterpret_cast<const double*>(&S.x0)[lane];
   } else if (warp == 2) {
@@ -867,6 +1094,7 @@ __device__ void gn_step_fast(const SolveParams& sp, Ctrl* c, FastSmem& S) {
     c->cost = sp.W_icp * S.sums[27] + sp.W_rgb * S.sums[kSums + 27] + S.cost;
     c->iterations += 1;
   }
+  return true;
 }
 
 // ---- the frame's constants (k_frame_begin) -----------------------------------------

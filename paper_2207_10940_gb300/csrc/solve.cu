@@ -745,18 +745,21 @@ __device__ void ldlt_solve_thread(const double* A, int n, int ld, double* b) {
 }
 
 // Pivot reciprocal: an FP32 seed refined by one Newton-Raphson step (relative
-// error below 2^-45; the factorisation is then exact for a matrix whose pivots
+// error below 2^-44.8; the factorisation is then exact for a matrix whose pivots
 // are perturbed by that amount, far below what the system's rounding already
-// costs).  The seed's conversions are integer operations on the bit patterns
-// (the leading 23 mantissa bits of d, the exponent re-biased between the
-// formats; d and 1 / d are normal in both here): on this GPU every FP64-pipe
-// instruction on the pivot's dependency chain costs tens of cycles.
+// costs).  The range test and the seed's conversions are integer operations on
+// the bit patterns (d rounded to 24 bits, the exponent re-biased between the
+// formats; d and 1 / d are normal in both here) and the seed itself is the
+// hardware's approximation: on this GPU every FP64-pipe instruction on the
+// pivot's dependency chain, a comparison included, costs 64 cycles.
 __device__ __forceinline__ double pivot_recip(double d) {
-  if (d > 1e-30 && d < 1e30) {
-    const int hi = __double2hiint(d);
+  const int hi = __double2hiint(d);
+  if ((unsigned)((hi >> 20) - (1023 - 99)) < 198u) {       // 2^-99 <= d < 2^99, positive
     const unsigned lo = (unsigned)__double2loint(d);
-    const float f = __int_as_float((int)(((unsigned)hi - 0x38000000u) << 3 | lo >> 29));
-    const int yb = __float_as_int(__frcp_rn(f));
+    const unsigned fb = (((unsigned)hi - 0x38000000u) << 3 | lo >> 29) + (lo >> 28 & 1u);
+    float y0;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(__uint_as_float(fb)));
+    const int yb = __float_as_int(y0);
     const double y = __hiloint2double((yb >> 3) + 0x38000000, (int)((unsigned)yb << 29));
     return fma(y, fma(-d, y, 1.0), y);
   }
@@ -1969,13 +1972,15 @@ __global__ void __launch_bounds__(kSolveThreads) k_linearise_end(SolveParams sp,
 __device__ int load_slot_params(const BatchArgs& a, SolveParams& sp) {
   const int slot = a.slot0 + blockIdx.x;
   const SlotDyn& d = batch_dyn(a, slot);
+  // the record and the parameters are loaded in one round; the per-launch fields
+  // (imu, level, last) are written by their own thread
+  constexpr int kFirst = offsetof(SolveParams, imu) / 4, kLast = offsetof(SolveParams, last) / 4;
   const int mode = d.mode;
-  if (mode == kSlotIdle) return mode;
   const uint32_t* src = reinterpret_cast<const uint32_t*>(&a.slots[slot].sp);
   uint32_t* dst = reinterpret_cast<uint32_t*>(&sp);
-  for (int i = threadIdx.x; i < (int)(sizeof(SolveParams) / 4); i += blockDim.x) dst[i] = src[i];
-  __syncthreads();
-  if (threadIdx.x == 0) {
+  for (int i = threadIdx.x; i < (int)(sizeof(SolveParams) / 4); i += blockDim.x)
+    if (i < kFirst || i > kLast) dst[i] = src[i];
+  if (threadIdx.x == blockDim.x - 1) {
     sp.imu = reinterpret_cast<const ImuHeader*>(a.dyn + d.imu_off);
     sp.level = a.level;
     sp.last = a.last;
@@ -2005,12 +2010,9 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_gn_step_batch(const BatchA
   } else if (mode == kSlotTrack) {
     // the covariance form, except where the full system is wanted (marginalisation
     // after the last iteration) or the frame's prior does not allow it
-    Ctrl* c = sp.ctrl;
-    if (!sp.last && sp.track_mode != DRI_TRACK_RGBD_ONLY && c->elim.ok) {
-      if (c->status == 0) gn_step_fast(sp, c, *reinterpret_cast<FastSmem*>(smem_raw));
-    } else {
+    if (sp.last || sp.track_mode == DRI_TRACK_RGBD_ONLY ||
+        !gn_step_fast(sp, *reinterpret_cast<FastSmem*>(smem_raw)))
       gn_step_body(sp, *reinterpret_cast<GnSmem*>(smem_raw));
-    }
   } else {
     grid_dep_wait();                    // idle slot: nothing to read, keep the ordering
   }
