@@ -266,11 +266,25 @@ inline int copy_tiles(int w, int h) {
 inline int map_tiles(int w, int h) {
   return ((w + kMapTileW - 1) / kMapTileW) * ((h + kMapTileH * kMapRows - 1) / (kMapTileH * kMapRows));
 }
-cudaError_t launch_normals(const LevelMaps& m, const Ctrl* ctrl, const LevelGeom& g,
-                           float dmin, float dmax, bool fp16, int which_set, cudaStream_t s);
-cudaError_t launch_gradient(const LevelMaps& m, const Ctrl* ctrl, int w, int h, bool fp16,
-                            cudaStream_t s);
-cudaError_t launch_track(const TrackParams& p, bool fp16, bool fp32_partials, cudaStream_t s);
+// The allocation-free pair entry: what its first kernel stores for the second
+// (transforms of the pixel kernel, zeroed counters) and what the second needs to
+// finish the systems in its last block.
+struct PairBegin {
+  Ctrl* ctrl;
+  uint32_t* counters;
+  int32_t ncounters;
+  float xf_icp[12], xf_rgb[12];
+};
+struct PairEnd {
+  double Rref[9], R0[9];
+  double W_icp, W_rgb;
+  dri_linearisation* out;
+};
+// normals of both sets, gradients of set 0, begin's record; flags (nullable) zeroed
+cudaError_t launch_pair_maps(const LevelMaps& m, const LevelGeom& g, float dmin, float dmax, bool fp16,
+                             const PairBegin& begin, uint8_t* flags, cudaStream_t s);
+cudaError_t launch_track(const TrackParams& p, const PairEnd& end, bool fp16, bool fp32_partials,
+                         cudaStream_t s);
 
 #ifdef __CUDACC__
 // Programmatic dependent launch between the batched pixel kernel and the

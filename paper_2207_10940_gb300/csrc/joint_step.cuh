@@ -471,11 +471,11 @@ __device__ void fast_gravity(FastSmem& S, bool gyro) {
     const double a[4] = {S.x0.qg[0], S.x0.qg[1], S.x0.qg[2], S.x0.qg[3]};
     double o = quat_mul_k(a, S.x1.qg, k, true);
     const double w = __shfl_sync(0xffffffffu, o, lane & ~3);
-    if (w < 0.0) o = -o;
+    if (__double2hiint(w) < 0) o = -o;
     double s2 = k ? o * o : 0.0;
     s2 += __shfl_xor_sync(0xffffffffu, s2, 1);
     s2 += __shfl_xor_sync(0xffffffffu, s2, 2);
-    const double f = quat_log_factor(s2, fabs(w));
+    const double f = pos_less(s2, 1e-6) ? 2.0 * fma(s2, fma(s2, 3.0 / 40, 1.0 / 6), 1.0) : quat_log_factor(s2, fabs(w));
     if (lane > 0 && lane < 4) S.eg[lane - 1] = f * o;
   }
   __syncwarp();
@@ -501,12 +501,11 @@ __device__ void fast_gravity(FastSmem& S, bool gyro) {
     v = gyro ? 0.0 : v * inv;
     if (lane < 2) S.a[lane] = v;
     else S.s = v, S.a[2] = 0.0;
-  } else if (lane < 9) {             // Gm row m, column k; det(B^T B) = |n|^2 (Lagrange's identity)
+  } else if (lane < 9) {             // Gm row m, column k; 1 / det(B^T B) = 1 / |n|^2 (Lagrange's identity)
     const int m = (lane - 3) / 3, k = (lane - 3) % 3;
-    const double det = fma(S.mm[0], S.mm[2], -(S.mm[1] * S.mm[1]));
     const double b0 = -B[3 * k], b1 = -B[3 * k + 1];
     const double v = m == 0 ? fma(S.mm[2], b0, -(S.mm[1] * b1)) : fma(S.mm[0], b1, -(S.mm[1] * b0));
-    S.Gm[3 * m + k] = gyro ? 0.0 : v / det;
+    S.Gm[3 * m + k] = gyro ? 0.0 : v * (inv * inv);
   }
   __syncwarp();
 }

@@ -12,8 +12,9 @@
 //
 // Depth and intensity are FP32 planes; the packs (packs.cuh) hold FP32 or, with
 // DRI_FP16_MAPS, FP16 normals and gradients.
-// The batched kernels cover the images of every slot of a plan in one launch;
-// the single-image normal and gradient kernels serve the allocation-free entry.
+// The batched kernels cover the images of every slot of a plan in one launch; the
+// pair kernel serves the allocation-free entry, the single-image gradient kernel an
+// uploaded reference.
 #include <cuda_fp16.h>
 
 #include "dri_internal.h"
@@ -193,13 +194,31 @@ __global__ void __launch_bounds__(256) k_gradient_batch(const BatchArgs a) {
     if (y < h) gradient_px<T>(tp.m, cs, w, h, x, y);
 }
 
+// Both images' normal maps and the reference's gradient map of the allocation-free
+// pair entry in one launch (as three, with a one-thread kernel of FP64 set-up in
+// front, their launches and that thread's chain were two thirds of the call).
 template <typename T>
-__global__ void k_normals(LevelMaps m, const Ctrl* __restrict__ ctrl, LevelGeom g, float dmin,
-                          float dmax, int which) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y * blockDim.y + threadIdx.y;
+__global__ void __launch_bounds__(256) k_pair_maps(LevelMaps m, LevelGeom g, float dmin, float dmax,
+                                                   PairBegin b, uint8_t* __restrict__ flags) {
+  grid_dep_launch();             // the pixel kernel waits for this grid's end itself
+  if (blockIdx.x == 0 && blockIdx.y == 0) {
+    const int t = threadIdx.y * 32 + threadIdx.x;
+    for (int i = t; i < b.ncounters; i += 256) b.counters[i] = 0u;
+    if (t < 12) b.ctrl->xf_icp[t] = b.xf_icp[t];
+    else if (t < 24) b.ctrl->xf_rgb[t - 12] = b.xf_rgb[t - 12];
+    else if (t == 24) {
+      b.ctrl->status = 0;
+      b.ctrl->ref_index = 0;
+      b.ctrl->margin_acc[0] = b.ctrl->margin_acc[1] = 0u;
+    }
+  }
+  const int x = blockIdx.x * 32 + threadIdx.x;
+  const int y = blockIdx.y * 8 + threadIdx.y;
   if (x >= g.w || y >= g.h) return;
-  normal_px<T>(m, which < 0 ? 1 - ctrl->ref_index : which, g, dmin, dmax, x, y);
+  normal_px<T>(m, 0, g, dmin, dmax, x, y);
+  normal_px<T>(m, 1, g, dmin, dmax, x, y);
+  gradient_px<T>(m, 0, g.w, g.h, x, y);
+  if (flags) flags[y * g.w + x] = 0;
 }
 
 template <typename T>
@@ -306,23 +325,11 @@ cudaError_t launch_gradient_batch(const BatchArgs& a, int blocks, bool fp16, cud
   return cudaGetLastError();
 }
 
-cudaError_t launch_normals(const LevelMaps& m, const Ctrl* ctrl, const LevelGeom& g, float dmin,
-                           float dmax, bool fp16, int which_set, cudaStream_t s) {
+cudaError_t launch_pair_maps(const LevelMaps& m, const LevelGeom& g, float dmin, float dmax, bool fp16,
+                             const PairBegin& begin, uint8_t* flags, cudaStream_t s) {
   const dim3 b(32, 8);
-  if (fp16)
-    k_normals<__half><<<grid2(g.w, g.h, b), b, 0, s>>>(m, ctrl, g, dmin, dmax, which_set);
-  else
-    k_normals<float><<<grid2(g.w, g.h, b), b, 0, s>>>(m, ctrl, g, dmin, dmax, which_set);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_gradient(const LevelMaps& m, const Ctrl* ctrl, int w, int h, bool fp16,
-                            cudaStream_t s) {
-  const dim3 b(32, 8);
-  if (fp16)
-    k_gradient<__half><<<grid2(w, h, b), b, 0, s>>>(m, ctrl, w, h);
-  else
-    k_gradient<float><<<grid2(w, h, b), b, 0, s>>>(m, ctrl, w, h);
+  if (fp16) k_pair_maps<__half><<<grid2(g.w, g.h, b), b, 0, s>>>(m, g, dmin, dmax, begin, flags);
+  else k_pair_maps<float><<<grid2(g.w, g.h, b), b, 0, s>>>(m, g, dmin, dmax, begin, flags);
   return cudaGetLastError();
 }
 

@@ -33,7 +33,6 @@
 #include <mutex>
 
 #include "dri_internal.h"
-#include "so3.cuh"
 
 namespace dri {
 namespace {
@@ -66,76 +65,21 @@ constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 void* g_scratch_addr[kMaxDevices] = {};
 
-// Per-call set-up: transforms of the pixel kernel from (x_ref, x0, x1) exactly as
-// the stream path computes them, status and counter cleared, set 0 = reference.
-__global__ void k_noalloc_begin(Ctrl* c, uint32_t* counters, DState xref, DState x0, DState x1) {
-  for (int i = threadIdx.x; i < 1 + kNoallocMaxGroups; i += blockDim.x) counters[i] = 0u;
-  if (threadIdx.x != 0) return;
-  double Rref[9], R0[9], R1[9], M[9], dr[3], t[3];
-  quat_to_rot(xref.q, Rref);
-  quat_to_rot(x0.q, R0);
-  quat_to_rot(x1.q, R1);
-  for (int i = 0; i < 9; ++i) c->Rref[i] = Rref[i];
-  for (int i = 0; i < 3; ++i) c->rref[i] = xref.r[i];
-  c->x0 = x0;
-  c->x1 = x1;
-  m3_tmul(Rref, R1, M);
-  for (int i = 0; i < 3; ++i) dr[i] = x1.r[i] - xref.r[i];
-  m3_tvec(Rref, dr, t);
-  for (int i = 0; i < 9; ++i) c->xf_icp[i] = (float)(M[i] - ((i % 4 == 0) ? 1.0 : 0.0));
-  for (int i = 0; i < 3; ++i) c->xf_icp[9 + i] = (float)t[i];
-  m3_tmul(R0, R1, M);
-  for (int i = 0; i < 3; ++i) dr[i] = x1.r[i] - x0.r[i];
-  m3_tvec(R0, dr, t);
-  for (int i = 0; i < 9; ++i) c->xf_rgb[i] = (float)(M[i] - ((i % 4 == 0) ? 1.0 : 0.0));
-  for (int i = 0; i < 3; ++i) c->xf_rgb[9 + i] = (float)t[i];
-  c->status = 0;
-  c->ref_index = 0;
-  c->block_counter = 0u;
-  c->margin_acc[0] = c->margin_acc[1] = 0u;
+// Rotation matrix of a unit quaternion, and the pixel kernel's transform
+// (A^T B - I, A^T d) in FP32 exactly as the stream path rounds it.
+void quat_to_rot_h(const double* q, double* R) {
+  const double w = q[0], x = q[1], y = q[2], z = q[3];
+  R[0] = 1 - 2 * (y * y + z * z); R[1] = 2 * (x * y - w * z);     R[2] = 2 * (x * z + w * y);
+  R[3] = 2 * (x * y + w * z);     R[4] = 1 - 2 * (x * x + z * z); R[5] = 2 * (y * z - w * x);
+  R[6] = 2 * (x * z - w * y);     R[7] = 2 * (y * z + w * x);     R[8] = 1 - 2 * (x * x + y * y);
 }
-
-// Weighted world-frame systems of both terms from the folded sums (the pixel
-// kernel works in the reference / x0 camera frames: H_W = Q H Q^T, Q = diag(R, R)).
-__global__ void k_noalloc_end(const Ctrl* c, double W_icp, double W_rgb, dri_linearisation* out) {
-  const int tid = threadIdx.x;
-  if (tid < 2 * 36) {
-    const int term = tid / 36, idx = tid % 36;
-    const int i = idx / 6, j = idx % 6;
-    double R[9];
-    if (term == 0) {
-      for (int k = 0; k < 9; ++k) R[k] = c->Rref[k];
-    } else {
-      quat_to_rot(c->x0.q, R);
+void transform_h(const double* A, const double* B, const double* d, float* xf) {
+  for (int i = 0; i < 3; ++i) {
+    for (int j = 0; j < 3; ++j) {
+      const double m = A[i] * B[j] + A[3 + i] * B[3 + j] + A[6 + i] * B[6 + j];
+      xf[3 * i + j] = (float)(m - (i == j ? 1.0 : 0.0));
     }
-    const double* s = c->sums + term * kSums;
-    auto hloc = [&](int a, int b) {
-      const int lo = a < b ? a : b, hi = a < b ? b : a;
-      return s[lo * 6 - lo * (lo - 1) / 2 + (hi - lo)];
-    };
-    double acc = 0.0;
-    const int bi = i / 3, ri = i % 3, bj = j / 3, rj = j % 3;
-    for (int k = 0; k < 3; ++k)
-      for (int l = 0; l < 3; ++l) acc += R[ri * 3 + k] * hloc(bi * 3 + k, bj * 3 + l) * R[rj * 3 + l];
-    const double w = term == 0 ? W_icp : W_rgb;
-    (term == 0 ? out->H_icp : out->H_rgb)[idx] = w * acc;
-    if (j == 0) {
-      double g = 0.0;
-      for (int k = 0; k < 3; ++k) g += R[ri * 3 + k] * s[21 + bi * 3 + k];
-      (term == 0 ? out->b_icp : out->b_rgb)[i] = -w * g;
-    }
-  }
-  for (int idx = tid; idx < 34 * 34; idx += blockDim.x) out->H[idx] = 0.0;
-  if (tid < 34) out->b[tid] = 0.0;
-  if (tid < 18) out->e_imu[tid] = 0.0;
-  if (tid == 0) {
-    out->cost_icp = W_icp * c->sums[27];
-    out->cost_rgb = W_rgb * c->sums[kSums + 27];
-    out->cost_imu = 0.0;
-    out->n_icp = (int64_t)c->sums[28];
-    out->n_rgb = (int64_t)c->sums[kSums + 28];
-    out->n_margin_icp = c->margin_acc[0];
-    out->n_margin_rgb = c->margin_acc[1];
+    xf[9 + i] = (float)(A[i] * d[0] + A[3 + i] * d[1] + A[6 + i] * d[2]);
   }
 }
 
@@ -236,12 +180,27 @@ extern "C" int dri_linearise_pair_noalloc(const dri_stream_config* cfg, const fl
   m.packB[1] = base + kOffPackB;                    // the live set's pack B is never read
 
   uint32_t* counters = reinterpret_cast<uint32_t*>(base + kOffCounters);
-  k_noalloc_begin<<<1, 32, 0, s>>>(ctrl, counters, dstate_of(*x_ref), dstate_of(*x0), dstate_of(*x1));
-  if (cudaGetLastError() != cudaSuccess) return DRI_ECUDA;
+  // transforms of the pixel kernel from (x_ref, x0, x1), as the stream path computes them
+  const DState dref = dstate_of(*x_ref), d0 = dstate_of(*x0), d1 = dstate_of(*x1);
+  PairBegin begin;
+  PairEnd end;
+  double R1[9], dr[3];
+  quat_to_rot_h(dref.q, end.Rref);
+  quat_to_rot_h(d0.q, end.R0);
+  quat_to_rot_h(d1.q, R1);
+  for (int i = 0; i < 3; ++i) dr[i] = d1.r[i] - dref.r[i];
+  transform_h(end.Rref, R1, dr, begin.xf_icp);
+  for (int i = 0; i < 3; ++i) dr[i] = d1.r[i] - d0.r[i];
+  transform_h(end.R0, R1, dr, begin.xf_rgb);
+  begin.ctrl = ctrl;
+  begin.counters = counters;
+  begin.ncounters = 1 + kNoallocMaxGroups;
+  end.W_icp = 1.0 / (cfg->sigma_d * cfg->sigma_d);
+  end.W_rgb = 1.0 / (cfg->sigma_I * cfg->sigma_I);
+  end.out = out;
   const float dmin = (float)cfg->depth_min, dmax = (float)cfg->depth_max;
-  if (launch_normals(m, ctrl, g, dmin, dmax, fp16, 0, s) != cudaSuccess) return DRI_ECUDA;
-  if (launch_normals(m, ctrl, g, dmin, dmax, fp16, 1, s) != cudaSuccess) return DRI_ECUDA;
-  if (launch_gradient(m, ctrl, g.w, g.h, fp16, s) != cudaSuccess) return DRI_ECUDA;
+  uint8_t* fl = flags ? base + kOffFlags : nullptr;
+  if (launch_pair_maps(m, g, dmin, dmax, fp16, begin, fl, s) != cudaSuccess) return DRI_ECUDA;
 
   TrackParams p;
   std::memset(&p, 0, sizeof(p));
@@ -251,7 +210,7 @@ extern "C" int dri_linearise_pair_noalloc(const dri_stream_config* cfg, const fl
   p.partials = base + kOffPartials;
   p.gpartials = base + kOffGPartials;
   p.counters = counters;
-  p.flags = flags ? base + kOffFlags : nullptr;
+  p.flags = fl;
   p.ppt = 1;
   p.nblocks = track_mixed_blocks(g.w, g.h, 1);
   if (p.nblocks > kNoallocMaxBlocks) return DRI_EINVAL;
@@ -261,12 +220,8 @@ extern "C" int dri_linearise_pair_noalloc(const dri_stream_config* cfg, const fl
   p.icp_cos = (float)std::cos(cfg->icp_angle_thr_deg * 3.14159265358979323846 / 180.0);
   p.occ_thr = (float)cfg->occlusion_thr;
   p.icp_dw = cfg->icp_depth_weight;
-  if (flags && cudaMemsetAsync(p.flags, 0, (size_t)g.w * g.h, s) != cudaSuccess) return DRI_ECUDA;
-  if (launch_track(p, fp16, fp32p, s) != cudaSuccess) return DRI_ECUDA;
+  if (launch_track(p, end, fp16, fp32p, s) != cudaSuccess) return DRI_ECUDA;
   if (flags && cudaMemcpyAsync(flags, p.flags, (size_t)g.w * g.h, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
     return DRI_ECUDA;
-  k_noalloc_end<<<1, 128, 0, s>>>(ctrl, 1.0 / (cfg->sigma_d * cfg->sigma_d),
-                                  1.0 / (cfg->sigma_I * cfg->sigma_I), out);
-  if (cudaGetLastError() != cudaSuccess) return DRI_ECUDA;
   return DRI_OK;
 }

@@ -420,6 +420,7 @@ __device__ __forceinline__ void rgb_rows(const TileCtx& c, float* acc, int& nm) 
   }
 }
 
+// (true in the block that folded the image's last group and wrote ctrl->sums)
 // One tile of one image (single-term: 32 x 8 * ppt pixels of `term`; mixed:
 // 32 x 4 * ppt pixels, warps 0-3 ICP and 4-7 photometric): (bx, by) its tile
 // coordinates, bid its index in the image's fold order.
@@ -428,10 +429,10 @@ __device__ __forceinline__ void rgb_rows(const TileCtx& c, float* acc, int& nm) 
 constexpr int kOptOcc = 1, kOptDepthWeight = 2;
 
 template <typename T, typename P, bool FLAGS, bool MARGIN, bool SPLIT, int OPT>
-__device__ __forceinline__ void track_tile(const TrackParams& p, const int term, const int bx,
+__device__ __forceinline__ bool track_tile(const TrackParams& p, const int term, const int bx,
                                            const int by, const int bid) {
   Ctrl* __restrict__ ctrl = p.ctrl;
-  if (ctrl->status != 0) return;
+  if (ctrl->status != 0) return false;
   const int lane = threadIdx.x;
   const int warp = threadIdx.y;
   const bool icp = SPLIT ? term == 0 : warp < kTrackRows;    // warp-uniform
@@ -538,7 +539,7 @@ __device__ __forceinline__ void track_tile(const TrackParams& p, const int term,
   __syncthreads();
   if (tid == 0) s_last = atomicAdd(&p.counters[1 + grp], 1u) == (unsigned)(gsize - 1);
   __syncthreads();
-  if (!s_last) return;
+  if (!s_last) return false;
   __threadfence();
   if (tid < kSumsAll) {
     P s = 0;
@@ -553,7 +554,7 @@ __device__ __forceinline__ void track_tile(const TrackParams& p, const int term,
     s_last = atomicAdd(&p.counters[0], 1u) == (unsigned)(ngroups - 1);
   }
   __syncthreads();
-  if (!s_last) return;
+  if (!s_last) return false;
   __threadfence();
   if (tid < kSumsAll) {
     P s = 0;
@@ -561,12 +562,58 @@ __device__ __forceinline__ void track_tile(const TrackParams& p, const int term,
     ctrl->sums[tid] = (double)s;
   }
   if (tid == 0) p.counters[0] = 0u;
+  return true;
+}
+
+// Weighted world-frame systems of both terms from the folded sums, by the block that
+// folded them (the pixel kernel works in the reference / x0 camera frames:
+// H_W = Q H Q^T, Q = diag(R, R)); the fields of the joint system are zeroed.
+__device__ void pair_end(const PairEnd& e, const Ctrl* c, int tid) {
+  dri_linearisation* out = e.out;
+  if (tid < 2 * 36) {
+    const int term = tid / 36, idx = tid % 36;
+    const int i = idx / 6, j = idx % 6;
+    const double* R = term == 0 ? e.Rref : e.R0;
+    const double* s = c->sums + term * kSums;
+    auto hloc = [&](int a, int b) {
+      const int lo = a < b ? a : b, hi = a < b ? b : a;
+      return s[lo * 6 - lo * (lo - 1) / 2 + (hi - lo)];
+    };
+    double acc = 0.0;
+    const int bi = i / 3, ri = i % 3, bj = j / 3, rj = j % 3;
+    for (int k = 0; k < 3; ++k)
+      for (int l = 0; l < 3; ++l) acc += R[ri * 3 + k] * hloc(bi * 3 + k, bj * 3 + l) * R[rj * 3 + l];
+    const double w = term == 0 ? e.W_icp : e.W_rgb;
+    (term == 0 ? out->H_icp : out->H_rgb)[idx] = w * acc;
+    if (j == 0) {
+      double g = 0.0;
+      for (int k = 0; k < 3; ++k) g += R[ri * 3 + k] * s[21 + bi * 3 + k];
+      (term == 0 ? out->b_icp : out->b_rgb)[i] = -w * g;
+    }
+  } else {
+    for (int idx = tid - 72; idx < 34 * 34; idx += 256 - 72) out->H[idx] = 0.0;
+    if (tid >= 128 && tid < 128 + 34) out->b[tid - 128] = 0.0;
+    if (tid >= 192 && tid < 192 + 18) out->e_imu[tid - 192] = 0.0;
+    if (tid == 255) {
+      out->cost_icp = e.W_icp * c->sums[27];
+      out->cost_rgb = e.W_rgb * c->sums[kSums + 27];
+      out->cost_imu = 0.0;
+      out->n_icp = (int64_t)c->sums[28];
+      out->n_rgb = (int64_t)c->sums[kSums + 28];
+      out->n_margin_icp = __ldcg(&c->margin_acc[0]);
+      out->n_margin_rgb = __ldcg(&c->margin_acc[1]);
+    }
+  }
 }
 
 template <typename T, typename P, bool FLAGS, int OPT>
 __global__ void __launch_bounds__(kTrackThreadsX * kTrackThreadsY)
-k_track(TrackParams p) {
-  track_tile<T, P, FLAGS, FLAGS, false, OPT>(p, 0, blockIdx.x, blockIdx.y, blockIdx.y * gridDim.x + blockIdx.x);
+k_track(TrackParams p, const __grid_constant__ PairEnd end) {
+  grid_dep_wait();               // the maps and transforms
+  if (track_tile<T, P, FLAGS, FLAGS, false, OPT>(p, 0, blockIdx.x, blockIdx.y, blockIdx.y * gridDim.x + blockIdx.x)) {
+    __syncthreads();             // ctrl->sums
+    pair_end(end, p.ctrl, threadIdx.y * kTrackThreadsX + threadIdx.x);
+  }
 }
 
 // Tiles of every tracking slot at one level: block -> (slot, tile, term)
@@ -622,18 +669,26 @@ int track_mixed_blocks(int w, int h, int ppt) {
   return gx * gy;
 }
 
-cudaError_t launch_track(const TrackParams& p0, bool fp16, bool fp32_partials, cudaStream_t s) {
+cudaError_t launch_track(const TrackParams& p0, const PairEnd& end, bool fp16, bool fp32_partials,
+                         cudaStream_t s) {
   TrackParams p = p0;
   p.nblocks = track_mixed_blocks(p.g.w, p.g.h, p.ppt);
-  const dim3 block(kTrackThreadsX, kTrackThreadsY);
   const int rows = kTrackRows * p.ppt;
-  const dim3 grid((p.g.w + kTrackThreadsX - 1) / kTrackThreadsX, (p.g.h + rows - 1) / rows);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((p.g.w + kTrackThreadsX - 1) / kTrackThreadsX, (p.g.h + rows - 1) / rows);
+  cfg.blockDim = dim3(kTrackThreadsX, kTrackThreadsY);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
   const bool flags = p.flags != nullptr;
   const int opt = (p.occ_thr > 0.f ? kOptOcc : 0) | (p.icp_dw ? kOptDepthWeight : 0);
 #define DRI_TRACK_OPT(T, P, O)                                              \
   do {                                                                      \
-    if (flags) k_track<T, P, true, O><<<grid, block, 0, s>>>(p);            \
-    else k_track<T, P, false, O><<<grid, block, 0, s>>>(p);                 \
+    if (flags) return cudaLaunchKernelEx(&cfg, k_track<T, P, true, O>, p, end); \
+    return cudaLaunchKernelEx(&cfg, k_track<T, P, false, O>, p, end);       \
   } while (0)
 #define DRI_TRACK_LAUNCH(T, P)                                              \
   do {                                                                      \
@@ -651,7 +706,6 @@ cudaError_t launch_track(const TrackParams& p0, bool fp16, bool fp32_partials, c
   }
 #undef DRI_TRACK_LAUNCH
 #undef DRI_TRACK_OPT
-  return cudaGetLastError();
 }
 
 cudaError_t launch_track_batch(const BatchArgs& a, int blocks, bool fp16, bool fp32_partials,
