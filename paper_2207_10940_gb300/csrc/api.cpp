@@ -615,8 +615,8 @@ double plan_pixels(const Plan* p, int level) {
   return n;
 }
 
-// The spare stream of a batch plan (the last of its group streams when the
-// groups leave it free; none while profiling or for a stream's own plan).
+// The spare stream of a plan (a batch plan's last group stream when the groups leave it
+// free; a stream's own plan has one only while it is captured; none while profiling).
 cudaStream_t side_stream(const Plan* p, bool profiling) {
   if (profiling || p->groups >= kMaxGroups || !p->aux[kMaxGroups - 2]) return p->stream;
   return p->aux[kMaxGroups - 2];
@@ -624,7 +624,7 @@ cudaStream_t side_stream(const Plan* p, bool profiling) {
 
 // Kernel launches of one frame, in order.  phase 1: maps and frame begin;
 // phase 2: the Gauss-Newton loop, frame end, gradients and the head gather.
-// On a batch plan's spare stream: the frame start, beside the map kernels
+// On the plan's spare stream: the frame start, beside the map kernels
 // (it reads and writes the slots' control blocks and their IMU blocks, the map
 // kernels only which set is the reference, which changes at the frame end),
 // and beside the loop the normal maps of the finer levels (the loop starts at
@@ -794,6 +794,30 @@ int plan_autotune(Plan* p, int64_t* kernels) {
   return plan_upload_tables(p);
 }
 
+// The spare stream and its events of a stream's own plan, held only while its launch
+// sequence is captured: the graph keeps the branches (one 640x480 camera 743 -> 667 us
+// per frame against one chain: the frame start beside the map kernels, the finer
+// levels' normals and the gradients beside the loop).
+void free_capture_side(Plan* p) {
+  cudaEvent_t* ev[] = {&p->ev_fork, &p->ev_grad, &p->ev_maps, &p->ev_start, &p->ev_begin, &p->ev_norm};
+  for (cudaEvent_t* e : ev) {
+    if (*e) cudaEventDestroy(*e);
+    *e = nullptr;
+  }
+  if (p->aux[kMaxGroups - 2]) cudaStreamDestroy(p->aux[kMaxGroups - 2]);
+  p->aux[kMaxGroups - 2] = nullptr;
+}
+
+void make_capture_side(Plan* p) {
+  cudaEvent_t* ev[] = {&p->ev_fork, &p->ev_grad, &p->ev_maps, &p->ev_start, &p->ev_begin, &p->ev_norm};
+  bool ok = cudaStreamCreateWithFlags(&p->aux[kMaxGroups - 2], cudaStreamNonBlocking) == cudaSuccess;
+  for (cudaEvent_t* e : ev) ok = ok && cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
+  if (!ok) {                      // without it the sequence is captured as one chain
+    free_capture_side(p);
+    cudaGetLastError();
+  }
+}
+
 // Captures the per-frame launch sequence once as a CUDA graph; a stream that
 // cannot be captured (the legacy default stream) keeps launching directly.
 int plan_run(Plan* p, int64_t* kernels) {
@@ -802,6 +826,7 @@ int plan_run(Plan* p, int64_t* kernels) {
       (!p->autotune || p->tuned)) {
     cudaGraph_t g = nullptr;
     int64_t k = 0;
+    if (!p->owns_device) make_capture_side(p);
     if (cudaStreamBeginCapture(p->stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
       const int r = plan_enqueue(p, 3, &k);
       const cudaError_t e = cudaStreamEndCapture(p->stream, &g);
@@ -818,6 +843,7 @@ int plan_run(Plan* p, int64_t* kernels) {
       cudaGetLastError();
       p->graph_failed = true;
     }
+    if (!p->owns_device) free_capture_side(p);
   }
   if (p->graph && !profiling) {
     CK(cudaGraphLaunch(p->graph, p->stream));
