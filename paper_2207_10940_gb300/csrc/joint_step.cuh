@@ -1096,6 +1096,103 @@ __device__ bool gn_step_fast(const SolveParams& sp, FastSmem& S) {
   return true;
 }
 
+// RGB-D-only baseline (DRI_TRACK_RGBD_ONLY): one Gauss-Newton step on x1's pose with
+// H_icp + lambda H_rgb (x1's blocks of the two pixel systems in W), x0 fixed; x1's
+// other components unchanged.  Whole block; what needs no pixel sum is done before the
+// wait for the pixel kernel, and the 6 x 6 system (27 entries with its right-hand side)
+// is swept by one warp without block barriers.  Against a block-wide factorisation
+// with FP64 divisions and a one-thread substitution: 18 -> 12 us per step (with its launch), 501x377 camera
+// 495 -> 362 us per frame.
+__device__ void gn_step_pose_only(const SolveParams& sp, FastSmem& S) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  Ctrl* c = sp.ctrl;
+  const int status = c->status;
+  if (tid < 20) reinterpret_cast<double*>(&S.x0)[tid] = reinterpret_cast<const double*>(&c->x0)[tid];
+  else if (tid < 40) reinterpret_cast<double*>(&S.x1)[tid - 20] = reinterpret_cast<const double*>(&c->x1)[tid - 20];
+  else if (tid >= 64 && tid < 73) S.Rref[tid - 64] = c->Rref[tid - 64];
+  else if (tid >= 73 && tid < 76) S.rref[tid - 73] = c->rref[tid - 73];
+  if (status != 0) return;
+  __syncthreads();
+  // C: diag(R0, R0) (photometric, rows 0-5) and diag(R_ref, R_ref) (ICP, rows 6-11)
+  if (tid < 9) S.R0[tid] = quat_rot_e(S.x0.q, tid);
+  __syncwarp();
+  if (warp == 0)
+    for (int idx = lane; idx < 72; idx += 32) {
+      const int i = idx / 6, k = idx - 6 * i, r = i % 6;
+      S.C[i][k] = r / 3 == k / 3 ? (i < 6 ? S.R0 : S.Rref)[3 * (r % 3) + k % 3] : 0.0;
+    }
+  grid_dep_wait();                    // the pixel sums
+  if (tid < kSumsAll) S.sums[tid] = __ldcg(c->sums + tid);
+  __syncthreads();
+  if (tid < 84) {                     // U = w C H_loc, and w C b_loc in column 6
+    const int i = tid / 7, q = tid - 7 * i, b = (i % 6) / 3 * 3;
+    const double* s = S.sums + (i < 6 ? kSums : 0);
+    double v = 0.0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const int lo = min(b + k, q), hi = max(b + k, q);
+      const double h = q == 6 ? s[21 + b + k] : s[lo * 6 - lo * (lo - 1) / 2 + (hi - lo)];
+      v = fma(S.C[i][b + k], h, v);
+    }
+    S.U[i][q] = v * (i < 6 ? sp.rgbd_lambda * sp.W_rgb : sp.W_icp);
+  }
+  __syncthreads();
+  if (warp == 0) {
+    int i = -1, j = -1;               // lower triangle by columns, then row 6: the right-hand side
+    double v = 0.0;
+    if (lane < 21) {
+      i = (int)((sqrtf(8.f * lane + 1.f) - 1.f) * 0.5f);
+      if (tri(i + 1, 0) <= lane) ++i;
+      if (tri(i, 0) > lane) --i;
+      j = lane - tri(i, 0);
+      const int b = j / 3 * 3;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) v = fma(S.U[i][b + k], S.C[j][b + k], fma(S.U[6 + i][b + k], S.C[6 + j][b + k], v));
+    } else if (lane < 27) {
+      i = 6;
+      j = lane - 21;
+      v = -(S.U[j][6] + S.U[6 + j][6]);
+    }
+    double rown = 0.0;
+#pragma unroll 1
+    for (int k = 0; k < 6; ++k) {
+      double* cb = S.col[k & 1];
+      *(j == k ? cb + i : S.sink + lane) = v;
+      __syncwarp();
+      const double t = cb[max(i, 0)] * cb[max(j, 0)];
+      const double r = pivot_recip(cb[k]);
+      const double w = fma(-t, r, v);
+      v = j > k ? w : v;
+      rown = j == k ? r : rown;
+    }
+    if (i > j) S.L[j][i] = v * rown;
+    bool good = !(i >= 0 && i == j) || (finite_bits(v) && v != 0.0 && __double2hiint(v) > 0);
+    __syncwarp();
+    const double* Lr = S.L[min(lane, 5)];
+    double y = Lr[6];
+#pragma unroll 1
+    for (int k = 5; k > 0; --k) y = fma(lane < k ? -Lr[k] : 0.0, __shfl_sync(0xffffffffu, y, k), y);
+    if (lane < 17) S.dx[lane] = lane < 6 ? y : 0.0;
+    good = __all_sync(0xffffffffu, good && (lane >= 6 || finite_bits(y)));
+    __syncwarp();
+    if (!good) {
+      if (lane == 0) c->status = DRI_ELOST;
+      return;
+    }
+    fast_boxplus(S.x1, S.dx);
+    fast_transforms(c, S);
+    if (lane < 20) reinterpret_cast<double*>(&c->x1)[lane] = reinterpret_cast<const double*>(&S.x1)[lane];
+    if (lane == 31) {
+      const double* s = S.sums;
+      c->n_icp[sp.level] = (int32_t)s[28];
+      c->n_rgb[sp.level] = (int32_t)s[kSums + 28];
+      store_margin(c, sp.level);
+      c->cost = sp.W_icp * s[27] + sp.rgbd_lambda * sp.W_rgb * s[kSums + 27];
+      c->iterations += 1;
+    }
+  }
+}
+
 // ---- the frame's constants (k_frame_begin) -----------------------------------------
 
 // Fills Ctrl::elim for the frame: the sweep operator over y (components 6..16) of

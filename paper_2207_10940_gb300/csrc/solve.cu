@@ -1294,52 +1294,6 @@ __device__ void assemble(const SolveParams& sp, GnSmem& S) {
   __syncthreads();
 }
 
-// RGB-D-only baseline (DRI_TRACK_RGBD_ONLY): one Gauss-Newton step on x1's pose
-// with H_icp + lambda H_rgb (x1's blocks of the two pixel systems in W), x0
-// fixed; 6x6 LDL^T; x1's other components unchanged.
-__device__ void gn_step_pose_only(const SolveParams& sp, GnSmem& S) {
-  Ctrl* c = sp.ctrl;
-  const int tid = threadIdx.x;
-  if (tid == 0) {
-    S.x0 = c->x0;
-    S.x1 = c->x1;
-  }
-  grid_dep_wait();                      // the pixel sums
-  if (tid >= 32 && tid < 32 + 2 * 36) pixel_system_entry(sp, c, S, tid - 32);
-  __syncthreads();
-  const double lam = sp.rgbd_lambda;
-  if (tid < 36) S.A[tid] = S.Hl[0][tid] + lam * S.Hl[1][tid];
-  else if (tid < 42) S.x[tid - 36] = S.gl[0][tid - 36] + lam * S.gl[1][tid - 36];
-  else if (tid < 53) S.x[tid - 36] = 0.0;                  // the other 11 tangent components
-  __syncthreads();
-  const bool pd = block_ldlt(S.A, 6, 6, S.col, &S.fail);
-  if (tid == 0) ldlt_solve_thread(S.A, 6, 6, S.x);
-  __syncthreads();
-  bool good = pd;
-  for (int i = 0; i < 6; ++i) good = good && isfinite(S.x[i]);
-  if (!good) {
-    if (tid == 0) c->status = DRI_ELOST;
-    return;
-  }
-  const int warp = tid >> 5;
-  if (warp == 0) {
-    warp_state_boxplus(S.x1, S.x);
-  } else if (tid == 64) {
-    const double* s = c->sums;
-    c->n_icp[sp.level] = (int32_t)s[28];
-    c->n_rgb[sp.level] = (int32_t)s[kSums + 28];
-    store_margin(c, sp.level);
-    c->cost = sp.W_icp * s[27] + lam * sp.W_rgb * s[kSums + 27];
-    c->iterations += 1;
-  }
-  __syncthreads();
-  if (warp == 0) {
-    warp_write_transforms(c, S.x0, S.x1, S.rot);
-  } else if (tid == 32) {
-    c->x1 = S.x1;
-  }
-}
-
 // Solver order of the reduced system: the 14 components no pixel term touches
 // (x0's velocity, biases and gravity, x1's velocity) first, then the 12 pose
 // components of x0 and x1 in the order of P12.  Reduced index of solver index s.
@@ -1358,10 +1312,6 @@ constexpr int kNonPose = 14;
 __device__ void gn_step_body(const SolveParams& sp, GnSmem& S) {
   Ctrl* c = sp.ctrl;
   if (c->status != 0) return;
-  if (sp.track_mode == DRI_TRACK_RGBD_ONLY) {
-    gn_step_pose_only(sp, S);
-    return;
-  }
   const int tid = threadIdx.x, nt = blockDim.x;
   assemble_state(sp, S);
   if (!S.ok) {
@@ -2010,8 +1960,9 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_gn_step_batch(const BatchA
   } else if (mode == kSlotTrack) {
     // the covariance form, except where the full system is wanted (marginalisation
     // after the last iteration) or the frame's prior does not allow it
-    if (sp.last || sp.track_mode == DRI_TRACK_RGBD_ONLY ||
-        !gn_step_fast(sp, *reinterpret_cast<FastSmem*>(smem_raw)))
+    if (sp.track_mode == DRI_TRACK_RGBD_ONLY)
+      gn_step_pose_only(sp, *reinterpret_cast<FastSmem*>(smem_raw));
+    else if (sp.last || !gn_step_fast(sp, *reinterpret_cast<FastSmem*>(smem_raw)))
       gn_step_body(sp, *reinterpret_cast<GnSmem*>(smem_raw));
   } else {
     grid_dep_wait();                    // idle slot: nothing to read, keep the ordering
