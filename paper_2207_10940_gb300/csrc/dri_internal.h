@@ -100,6 +100,9 @@ struct Ctrl {
   double pre_lin[61];
   double b_lin[6];
   Elim elim;
+  DState xl0, xl1;                    // where the running iteration linearises
+  int32_t lin_split;                  // 1: H, b hold the last system without its pixel terms
+  int32_t pad2;
 };
 
 // Bytes of the result head (x .. pad1) copied back after each frame.

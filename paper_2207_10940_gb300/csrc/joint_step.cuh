@@ -1,6 +1,7 @@
 // The Gauss-Newton step of the joint problem with the non-pose unknowns
-// eliminated in covariance form (Eq. 6-7), for every iteration of a frame but
-// its last (which assembles the full system that marginalisation takes).
+// eliminated in covariance form (Eq. 6-7).  The full system that marginalisation
+// takes is assembled beside a frame's last step, at the same linearisation point,
+// by a second block (step_lin_block in solve.cu).
 //
 // What bounds a step is the FP64 pipe: on GB300 a warp's FP64 instruction holds
 // its sub-partition's pipe for 64 cycles whatever the number of active lanes
@@ -54,7 +55,15 @@ constexpr int kNode = 61;             // odd stride: consecutive nodes fall into
 constexpr int kLam = 7, kPose = 12, kSys = kLam + kPose;      // 19 unknowns of the sweep
 constexpr int kSysEnt = kSys * (kSys + 1) / 2 + kSys;         // lower triangle + right-hand side row
 
-struct FastSmem {
+// The pixel terms of the joint system.
+struct PixSmem {
+  double C[18][6];                    // Jacobian maps: photometric on (p0, p1), ICP on p1
+  double sums[kSumsAll];
+  double U[18][7];
+  double P12[kPose * kPose], g12[kPose];   // lower triangle
+};
+
+struct FastSmem : PixSmem {
   double nodeA[kElimPieces][kNode];   // leaves, then every second level of the tree
   double nodeB[kElimPieces / 2][kNode];
   double X[kElimPieces / 2][18];      // V_2 - [v_2]x Phi_1 and P_2 - [p_2]x Phi_1 of each pair
@@ -70,7 +79,6 @@ struct FastSmem {
   double d[17], m[11], bp[6];         // x0 boxminus xbar; mean of y; prior vector on p0
   double eg[3], Jlg[9], Jrg[9], nv[3], mm[3], a[3], s, Gm[6], Ag[6];
   double eb[6];                       // bias errors
-  double C[18][6];                    // pixel Jacobian maps: photometric on (p0, p1), ICP on p1
   // after the pre-integration
   double Jyr[3][11];                  // position rows by y
   double RW[9], APg[9], t3[3], M[9], RP[9], t4[3], u[3], er[3], ea[3], Jla[9], B13[9];
@@ -79,10 +87,6 @@ struct FastSmem {
   double Jp[kLam][kPose];             // J'
   double ep[kLam];                    // e'
   double S[28];                       // S's lower triangle (without blockdiag(S6, sigma_g^2))
-  // pixel terms
-  double sums[kSumsAll];
-  double U[18][7];
-  double P12[kPose * kPose], g12[kPose];
   // sweep
   double col[2][kSys + 1];
   double sink[128];                   // where a lane without a value to publish writes
@@ -323,6 +327,7 @@ __device__ const double* fast_first_order(const SolveParams& sp, Ctrl* c, FastSm
     bar_sync<1, 128>();                          // every thread has read b_lin
     fast_leaves(S, np, bg, ba);
     const double* n = fast_tree(S, np);
+    if (sp.last) return n;                       // nobody uses the point any more; a reader may run beside
     if (t < 60) {
       const int src = t < 9 ? kNR + t : t < 15 ? kNv + t - 9 : kNPhi + t - 15;   // Phi, V, P, Va, Pa follow
       c->pre_lin[t] = n[src];
@@ -404,6 +409,20 @@ __device__ __forceinline__ double fast_jlinv_e(const double* w0, double s, int e
   return fma(c, fma(w[r], w[q], r == q ? -t2 : 0.0), fma(-0.5, hat_e(w, e), r == q ? 1.0 : 0.0));
 }
 
+// C of the pixel terms by one warp: the photometric local Jacobian on p0,
+// -[R0 0; [dr]x R0, R0] with dr = r1 - r0, and on p1, diag(R0, R0); the ICP one on p1,
+// diag(R_ref, R_ref).
+__device__ __forceinline__ void fill_pixel_maps(PixSmem& S, const double* R0, const double* Rref, const double* dr) {
+  const int lane = threadIdx.x & 31;
+  for (int idx = lane; idx < 108; idx += 32) {
+    const int i = idx / 6, k = idx - 6 * i, b = i / 3, r = i - 3 * b, kb = k / 3, q = k - 3 * kb;
+    double v = 0.0;
+    if ((b & 1) == kb) v = b < 2 ? -R0[3 * r + q] : b < 4 ? R0[3 * r + q] : Rref[3 * r + q];
+    if (!(b == 1 && kb == 0)) S.C[i][k] = v;
+  }
+  if (lane < 9) S.C[3 + lane / 3][lane % 3] = -hatm_e(dr, R0, lane);
+}
+
 // Rotations of the states and everything that needs them only; warp 5.
 __device__ void fast_state_terms(const SolveParams& sp, FastSmem& S) {
   const int lane = threadIdx.x & 31, g3 = lane / 9, e9 = lane - 9 * g3;
@@ -432,31 +451,20 @@ __device__ void fast_state_terms(const SolveParams& sp, FastSmem& S) {
     S.Jyr[r3][c3] = T * S.Q0[3 * c3 + r3];                    // position by velocity: T Q0^T
   }
   __syncwarp();
-  double hr = 0.0;
   if (lane < 9) {                    // position by gravity: Q0^T [c]x, first two columns
     const double v = mhat_e(S.Q0, true, S.c, lane);
     if (lane % 3 < 2) S.Jyr[lane / 3][9 + lane % 3] = v;
-  } else if (lane < 18) {
-    hr = hatm_e(S.dr, S.R0, e9);     // [r1 - r0]x R0
-  } else if (lane < 21) {
+  } else if (lane >= 18 && lane < 21) {
     const int i = lane - 18;
     S.base[i] = ((S.x0.r[i] + S.t1[i]) + S.t2c[i]) - S.x1.r[i];
-  } else if (lane < 27) {
+  } else if (lane >= 21 && lane < 27) {
     const int i = lane - 21;
     S.eb[i] = i < 3 ? S.x0.bg[i] - S.x1.bg[i] : S.x0.ba[i - 3] - S.x1.ba[i - 3];
-  } else if (lane < 30) {
+  } else if (lane >= 27 && lane < 30) {
     const int i = lane - 27;         // velocity error without its pre-integrated part
     S.evb[i] = fma(i == 2 ? -sp.g : 0.0, T, S.x0.v[i]) - S.x1.v[i];
   }
-  // C: the photometric local Jacobian on p0, -[R0 0; [dr]x R0, R0], and on p1,
-  // diag(R0, R0); the ICP one on p1, diag(R_ref, R_ref)
-  for (int idx = lane; idx < 108; idx += 32) {
-    const int i = idx / 6, k = idx - 6 * i, b = i / 3, r = i - 3 * b, kb = k / 3, q = k - 3 * kb;
-    double v = 0.0;
-    if ((b & 1) == kb) v = b < 2 ? -S.R0[3 * r + q] : b < 4 ? S.R0[3 * r + q] : S.Rref[3 * r + q];
-    if (!(b == 1 && kb == 0)) S.C[i][k] = v;
-  }
-  if (lane >= 9 && lane < 18) S.C[3 + e9 / 3][e9 % 3] = -hr;
+  fill_pixel_maps(S, S.R0, S.Rref, S.dr);
   __syncwarp();
 }
 
@@ -533,7 +541,7 @@ __device__ void fast_prior(FastSmem& S, bool gyro) {
 // ---- the pixel terms (warps 4-7) ------------------------------------------------
 
 // P12 (lower triangle) and g12: U = w C H_loc for both terms, then U C^T.
-__device__ void fast_pixel_terms(const SolveParams& sp, const Ctrl* c, FastSmem& S) {
+__device__ void fast_pixel_terms(const SolveParams& sp, const Ctrl* c, PixSmem& S) {
   const int t = threadIdx.x - 128;
   if (t < kSumsAll) S.sums[t] = __ldcg(c->sums + t);
   bar_sync<3, 128>();
@@ -1086,6 +1094,12 @@ __device__ bool gn_step_fast(const SolveParams& sp, FastSmem& S) {
     if (lane < 20) reinterpret_cast<double*>(&c->x0)[lane] = reinterpret_cast<const double*>(&S.x0)[lane];
   } else if (warp == 2) {
     if (lane < 20) reinterpret_cast<double*>(&c->x1)[lane] = reinterpret_cast<const double*>(&S.x1)[lane];
+  } else if (warp >= 4 && !sp.last) { // the next iteration's linearisation point
+    if (tid < 148) reinterpret_cast<double*>(&c->xl0)[tid - 128] = reinterpret_cast<const double*>(&S.x0)[tid - 128];
+    else if (tid < 168) reinterpret_cast<double*>(&c->xl1)[tid - 148] = reinterpret_cast<const double*>(&S.x1)[tid - 148];
+  } else if (warp >= 4) {             // what the marginalisation needs of the last iteration
+    if (tid < 162) c->d[tid - 128] = S.dx[tid - 128];
+    else if (tid == 162) c->lin_split = 1;
   } else if (tid == 96) {
     c->n_icp[sp.level] = (int32_t)S.sums[28];
     c->n_rgb[sp.level] = (int32_t)S.sums[kSums + 28];

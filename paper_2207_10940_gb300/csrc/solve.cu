@@ -907,10 +907,11 @@ __device__ void store_lin(Ctrl* c, const Preint& P, const double* bg, const doub
 //   dp = dp_lin + P_g dbg + P_a dba,  Phi_g <- Jr(Phi_g dbg) Phi_g
 // (the rotation's bias Jacobian at the updated point; the others are linear).
 // Once |dbg| > relin_g or |dba| > relin_a the samples are re-integrated at
-// (bg, ba), which become the linearisation point.  Whole block; P in shared
+// (bg, ba), which become the linearisation point (move_point).  Whole block; P in shared
 // memory; `scratch` 19 doubles of shared memory.
 __device__ bool preint_first_order(const SolveParams& sp, Ctrl* c, const double* bg,
-                                   const double* ba, ImuWork& W, Preint& P, double* scratch) {
+                                   const double* ba, ImuWork& W, Preint& P, double* scratch,
+                                   bool move_point) {
   const int tid = threadIdx.x;
   double dbg[3], dba[3];
 #pragma unroll
@@ -922,7 +923,7 @@ __device__ bool preint_first_order(const SolveParams& sp, Ctrl* c, const double*
   const double na = sqrt(dba[0] * dba[0] + dba[1] * dba[1] + dba[2] * dba[2]);
   if (ng > sp.relin_g || na > sp.relin_a) {      // uniform over the block
     const bool ok = preintegrate_block(sp.imu, bg, ba, false, 0.0, 0.0, W, P);
-    if (ok) store_lin(c, P, bg, ba);
+    if (ok && move_point) store_lin(c, P, bg, ba);
     return ok;
   }
   const double* L = c->pre_lin;
@@ -1060,24 +1061,24 @@ __device__ void pixel_system_entry(const SolveParams& sp, const Ctrl* c, Smem& S
 
 
 // State-only part of the joint system (Eq. 7 without the pixel terms) at
-// (ctrl->x0, ctrl->x1): the IMU term (Eq. 5-6), the prior on x0, and the
-// reduced system with x1's biases and gravity eliminated in closed form.
+// (x0, x1): the IMU term (Eq. 5-6), the prior on x0, and the reduced system with x1's biases and gravity eliminated in closed form.
 // Whole block.  Reads no pixel sum, so it runs while the preceding pixel kernel
 // is still at work.  Leaves the upper triangle of the full 34-dimensional S.H,
 // S.b, the reduced 26-dimensional S.Hr (full), S.br, and S.cost_imu; S.ok false
 // (in every thread) if the IMU samples do not cover the interval.
-__device__ void assemble_state(const SolveParams& sp, GnSmem& S) {
+__device__ void assemble_state(const SolveParams& sp, GnSmem& S, const DState& x0, const DState& x1,
+                               bool move_point = true) {
   Ctrl* c = sp.ctrl;
   const int tid = threadIdx.x, nt = blockDim.x;
   if (tid == 0) {
-    S.x0 = c->x0;
-    S.x1 = c->x1;
+    S.x0 = x0;
+    S.x1 = x1;
   }
   if ((tid >> 5) == 4) {
-    warp_state_boxminus(c->x0, c->xbar, S.dprior);
+    warp_state_boxminus(x0, c->xbar, S.dprior);
   } else if (tid == 160) {
     for (int i = 0; i < 36; ++i) S.M6[i] = (i % 7 == 0) ? 1.0 : 0.0;
-    const double d[3] = {c->x1.r[0] - c->x0.r[0], c->x1.r[1] - c->x0.r[1], c->x1.r[2] - c->x0.r[2]};
+    const double d[3] = {x1.r[0] - x0.r[0], x1.r[1] - x0.r[1], x1.r[2] - x0.r[2]};
     double K[9];
     hat3(d, K);
     for (int r = 0; r < 3; ++r)
@@ -1085,7 +1086,7 @@ __device__ void assemble_state(const SolveParams& sp, GnSmem& S) {
   }
   __syncthreads();
   S.ok = sp.imu_mode == DRI_IMU_FIRST_ORDER
-             ? preint_first_order(sp, c, S.x0.bg, S.x0.ba, S.W, S.P, S.fo)
+             ? preint_first_order(sp, c, S.x0.bg, S.x0.ba, S.W, S.P, S.fo, move_point)
              : preintegrate_block(sp.imu, S.x0.bg, S.x0.ba, false, 0.0, 0.0, S.W, S.P);
   if (!S.ok) return;
   imu_linearise(S.x0, S.x1, S.P, sp, S.L, S.J);
@@ -1280,7 +1281,7 @@ __device__ void add_pixel_terms(GnSmem& S, int t, int n) {
 // S.Hl, S.gl and S.cost_imu (dri_linearise).
 __device__ void assemble(const SolveParams& sp, GnSmem& S) {
   const int tid = threadIdx.x, nt = blockDim.x;
-  assemble_state(sp, S);
+  assemble_state(sp, S, sp.ctrl->x0, sp.ctrl->x1);
   if (!S.ok) return;
   grid_dep_wait();
   if (tid < 128) pixel_terms<3>(sp, S, tid);
@@ -1313,7 +1314,7 @@ __device__ void gn_step_body(const SolveParams& sp, GnSmem& S) {
   Ctrl* c = sp.ctrl;
   if (c->status != 0) return;
   const int tid = threadIdx.x, nt = blockDim.x;
-  assemble_state(sp, S);
+  assemble_state(sp, S, sp.ctrl->x0, sp.ctrl->x1);
   if (!S.ok) {
     if (tid == 0) c->status = DRI_ENOTREADY;
     return;
@@ -1460,7 +1461,7 @@ __device__ void gn_step_g3(const SolveParams& sp, Gn3Smem& S) {
   }
   __syncthreads();
   S.ok = sp.imu_mode == DRI_IMU_FIRST_ORDER
-             ? preint_first_order(sp, c, S.x0.bg, S.x0.ba, S.W, S.P, S.fo)
+             ? preint_first_order(sp, c, S.x0.bg, S.x0.ba, S.W, S.P, S.fo, true)
              : preintegrate_block(sp.imu, S.x0.bg, S.x0.ba, false, 0.0, 0.0, S.W, S.P);
   if (!S.ok) {
     if (tid == 0) c->status = DRI_ENOTREADY;
@@ -1733,6 +1734,7 @@ __device__ void frame_begin_body(const SolveParams& sp, BeginSmem& B) {
     c->cost = 0.0;
     for (int l = 0; l < kMaxLevels; ++l) c->n_icp[l] = c->n_rgb[l] = c->n_margin[l] = 0;
     c->margin_acc[0] = c->margin_acc[1] = 0u;
+    c->lin_split = 0;
   }
   __syncthreads();
   if (sp.track_mode == DRI_TRACK_RGBD_ONLY) {     // x1 starts at x0; no IMU term
@@ -1747,89 +1749,196 @@ __device__ void frame_begin_body(const SolveParams& sp, BeginSmem& B) {
   }
   const bool ok = imu_weight_and_prediction(sp, c, B, &c->x1);
   if (ok && (tid >> 5) == 0) warp_write_transforms(c, c->x0, c->x1, B.rot);
+  if (ok && tid >= 32 && tid < 52) {              // the first iteration's linearisation point
+    reinterpret_cast<double*>(&c->xl0)[tid - 32] = reinterpret_cast<const double*>(&c->x0)[tid - 32];
+    reinterpret_cast<double*>(&c->xl1)[tid - 32] = reinterpret_cast<const double*>(&c->x1)[tid - 32];
+  }
 }
 
-// NS: tangent dimension of a state (17, or 18 for the 3-D gravity form).
-template <int NS>
-__device__ void frame_end_body(const SolveParams& sp) {
-  constexpr int NJ = 2 * NS;
+// The state-only part of the joint system at the last iteration's linearisation point
+// (c->xl0, c->xl1), for the marginalisation: a block of its own beside the step's, whose
+// covariance form does not produce it.  Nothing it reads is written by that step (the
+// first-order update's linearisation point does not move in a frame's last step).
+__device__ void step_lin_block(const SolveParams& sp, GnSmem& S) {
   Ctrl* c = sp.ctrl;
   const int tid = threadIdx.x;
-  __shared__ int s_ok, s_fail;
-  if (tid == 0) {
-    if (c->status == 0 && c->n_icp[0] + c->n_rgb[0] < sp.min_valid) c->status = DRI_ELOST;
-    s_ok = c->status == 0;
+  if (c->status != 0 || !c->elim.ok) return;
+  assemble_state(sp, S, c->xl0, c->xl1, false);
+  if (!S.ok) return;                  // the step itself reports it
+  for (int idx = tid; idx < 34 * 34; idx += kSolveThreads) {
+    const int i = idx / 34, j = idx % 34;
+    c->H[idx] = j >= i ? S.H[idx] : S.H[j * 34 + i];
   }
-  __syncthreads();
-  if (!s_ok) {
-    if (tid == 0) c->x = c->xstart;
-    return;
-  }
-  if (sp.track_mode == DRI_TRACK_RGBD_ONLY) {     // no prior to carry over
-    if (tid == 0) {
-      c->x = c->x1;
-      c->xbar = c->x1;
-      c->t_state = sp.imu->t1;
-      load_pose_ref(c);
-      c->ref_index = 1 - c->ref_index;
+  if (tid < 34) c->b[tid] = S.b[tid];
+}
+
+struct EndSmem : PixSmem {
+  double H[36 * 36];
+  double b[36], d[36], bp[36];
+  double col[2][40];
+  double R0[9], Rref[9], dr[3];
+  int ok, bad;
+};
+
+// Reciprocal of a positive pivot to FP64 rounding (two Newton steps): the
+// marginalisation subtracts large terms (the IMU weights) from one another.
+__device__ __forceinline__ double pivot_recip_full(double d) {
+  const double y = pivot_recip(d);
+  return fma(y, fma(-d, y, 1.0), y);
+}
+
+// Schur complement (Eq. 8) of the leading NS x NS block of [H | bp] (row-major 2 NS,
+// full) onto the trailing one: element-parallel elimination on warps 0-3, an entry of
+// the lower triangle and of the right-hand side row per thread and slot, entries dealt
+// out by how long they are updated (the trailing block through all NS pivots), so that
+// a slot of a warp is done when its first entry is.  Writes H*, b* (hold: components
+// left without information).  False (in those threads) if a pivot is not positive.
+template <int NS>
+__device__ bool eliminate_x0(EndSmem& E, Ctrl* c, bool gyro) {
+  constexpr int NJ = 2 * NS, kTrail = NS * (NS + 1) / 2 + NS;
+  constexpr int kEnt = kTrail + NS * (NS + 2) + NS * (NS - 1) / 2;
+  constexpr int kOwn = (kEnt + 127) / 128;
+  const int t = threadIdx.x;
+  int ei[kOwn], ej[kOwn], life[kOwn];
+  double v[kOwn];
+#pragma unroll
+  for (int o = 0; o < kOwn; ++o) {
+    const int e = t + 128 * o;
+    int i = -1, j = -1, l = 0;
+    if (e < kTrail) {
+      i = (int)((sqrtf(8.f * e + 1.f) - 1.f) * 0.5f);
+      if (tri(i + 1, 0) <= e) ++i;
+      if (tri(i, 0) > e) --i;
+      j = NS + e - tri(i, 0);
+      i += NS;                        // row NJ: the right-hand side
+      l = NS;
+    } else if (e < kEnt) {            // column j = NS - 1 - g holds rows j .. NJ: NS + 2 + g entries
+      int f = e - kTrail, g = 0;
+      while (f >= NS + 2 + g) f -= NS + 2 + g++;
+      j = NS - 1 - g;
+      i = j + f;
+      l = j;
     }
-    return;
+    ei[o] = i;
+    ej[o] = j;
+    life[o] = __shfl_sync(0xffffffffu, l, 0);
+    v[o] = i < 0 ? 0.0 : i == NJ ? E.bp[j] : E.H[i * NJ + j];
   }
-  // b' = b - H d; Schur complement of the x0 block (Eq. 8)
-  __shared__ double H[NJ * NJ];
-  __shared__ double bp[NJ];
-  __shared__ double L[NS * NS];
-  __shared__ double X[NS * (NS + 1)];
-  __shared__ double colbuf[NJ];
-  __shared__ double Hs[NS * NS], bs[NS];
-  for (int idx = tid; idx < NJ * NJ; idx += blockDim.x) H[idx] = c->H[idx];
-  __syncthreads();
+  bool good = true;
+#pragma unroll 1
+  for (int k = 0; k < NS; ++k) {
+    double* cb = E.col[k & 1];
+#pragma unroll
+    for (int o = 0; o < kOwn; ++o)
+      if (ej[o] == k) cb[ei[o]] = v[o];
+    bar_sync<1, 128>();
+    const double d = cb[k];
+    good = good && __double2hiint(d) > 0 && finite_bits(d);
+    const double r = pivot_recip_full(d);
+#pragma unroll
+    for (int o = 0; o < kOwn; ++o)
+      if (life[o] > k) {              // uniform over the warp
+        const double w = fma(-(cb[max(ei[o], 0)] * r), cb[max(ej[o], 0)], v[o]);
+        v[o] = ej[o] > k ? w : v[o];
+      }
+  }
+  if (!good) return false;
+#pragma unroll
+  for (int o = 0; o < kOwn; ++o) {
+    const int i = ei[o] - NS, j = ej[o] - NS;
+    if (j < 0) continue;
+    if (i == NS) {
+      c->bs[j] = gyro && held_gyro_only(j) ? 0.0 : v[o];
+    } else {
+      const double h = gyro && (held_gyro_only(i) || held_gyro_only(j)) ? 0.0 : v[o];
+      c->Hs[i * NS + j] = h;
+      c->Hs[j * NS + i] = h;
+    }
+  }
+  return true;
+}
+
+// NS: tangent dimension of a state (17, or 18 for the 3-D gravity form).  The last
+// iteration's system, moved to the updated point (b <- b - H d), loses x0 (Eq. 8); the
+// frame becomes the reference.  Against a block-wide LDL^T with FP64 divisions and 18
+// one-thread substitutions, and the last system assembled beside the step
+// instead of by it: one 640x480 camera 657 -> 639 us per frame, 320x240 571 -> 536.
+template <int NS>
+__device__ void frame_end_body(const SolveParams& sp, EndSmem& E) {
+  constexpr int NJ = 2 * NS;
+  Ctrl* c = sp.ctrl;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int status = c->status, found = c->n_icp[0] + c->n_rgb[0], split = c->lin_split;
+  for (int idx = tid; idx < NJ * NJ; idx += kSolveThreads) E.H[idx] = c->H[idx];
   if (tid < NJ) {
-    double acc = c->b[tid];
-    for (int k = 0; k < NJ; ++k) acc -= H[tid * NJ + k] * c->d[k];
-    bp[tid] = acc;
+    E.b[tid] = c->b[tid];
+    E.d[tid] = c->d[tid];
   }
-  for (int idx = tid; idx < NS * NS; idx += blockDim.x) L[idx] = H[(idx / NS) * NJ + idx % NS];
-  __syncthreads();
-  const bool pd = block_ldlt(L, NS, NS, colbuf, &s_fail);
-  if (tid < NS + 1) {
-    double colv[NS];
-    for (int i = 0; i < NS; ++i) colv[i] = tid < NS ? H[i * NJ + NS + tid] : bp[i];
-    ldlt_solve_thread(L, NS, NS, colv);
-    for (int i = 0; i < NS; ++i) X[i * (NS + 1) + tid] = colv[i];
+  if (tid == 0) {
+    E.ok = status == 0 && found >= sp.min_valid;
+    if (status == 0 && !E.ok) c->status = DRI_ELOST;
   }
   __syncthreads();
-  for (int idx = tid; idx < NS * NS; idx += blockDim.x) {
-    const int i = idx / NS, j = idx % NS;
-    double acc = H[(NS + i) * NJ + NS + j];
-    for (int k = 0; k < NS; ++k) acc -= H[(NS + i) * NJ + k] * X[k * (NS + 1) + j];
-    Hs[idx] = acc;
-  }
-  if (tid < NS) {
-    double acc = bp[NS + tid];
-    for (int k = 0; k < NS; ++k) acc -= H[(NS + tid) * NJ + k] * X[k * (NS + 1) + NS];
-    bs[tid] = acc;
-  }
-  __syncthreads();
-  if (!pd) {
-    if (tid == 0) {
-      c->status = DRI_ELOST;
-      c->x = c->xstart;
-    }
+  if (!E.ok) {
+    if (tid < 20) reinterpret_cast<double*>(&c->x)[tid] = reinterpret_cast<const double*>(&c->xstart)[tid];
     return;
   }
-  // no information on held parts (gyro-only, 2-DoF form only)
-  const bool gyro = NS == 17 && sp.track_mode == DRI_TRACK_GYRO_ONLY;
-  for (int idx = tid; idx < NS * NS; idx += blockDim.x) {
-    const int i = idx / NS, j = idx % NS;
-    c->Hs[idx] = gyro && (held_gyro_only(i) || held_gyro_only(j)) ? 0.0 : 0.5 * (Hs[i * NS + j] + Hs[j * NS + i]);
+  if (sp.track_mode != DRI_TRACK_RGBD_ONLY) {     // the baseline has no prior to carry over
+    if (NS == 17 && split) {          // the pixel terms at the last linearisation point
+      if (warp >= 4) {
+        if (warp == 4) {
+          if (lane < 9) {
+            E.R0[lane] = quat_rot_e(c->xl0.q, lane);
+            E.Rref[lane] = c->Rref[lane];
+          } else if (lane < 12) {
+            E.dr[lane - 9] = c->xl1.r[lane - 9] - c->xl0.r[lane - 9];
+          }
+          __syncwarp();
+          fill_pixel_maps(E, E.R0, E.Rref, E.dr);
+        }
+        bar_sync<3, 128>();
+        fast_pixel_terms(sp, c, E);
+      }
+      __syncthreads();
+      if (tid < 144) {
+        const int i = tid / 12, j = tid - 12 * i;
+        E.H[pose_coord(i) * NJ + pose_coord(j)] += E.P12[max(i, j) * kPose + min(i, j)];
+      } else if (tid < 156) {
+        E.b[pose_coord(tid - 144)] += E.g12[tid - 144];
+      }
+      __syncthreads();
+    }
+    if (tid < 4 * NJ) {               // b' = b - H d, four lanes per row
+      const int i = tid >> 2, q = tid & 3;
+      const unsigned m = __activemask();
+      double v = 0.0;
+      for (int k = q; k < NJ; k += 4) v = fma(-E.H[i * NJ + k], E.d[k], v);
+      v += __shfl_xor_sync(m, v, 1);
+      v += __shfl_xor_sync(m, v, 2);
+      if (q == 0) E.bp[i] = E.b[i] + v;
+    }
+    __syncthreads();
+    if (warp < 4) {
+      const bool pd = eliminate_x0<NS>(E, c, NS == 17 && sp.track_mode == DRI_TRACK_GYRO_ONLY);
+      if (tid == 0) E.bad = !pd;
+    }
+    __syncthreads();
+    if (E.bad) {
+      if (tid == 0) c->status = DRI_ELOST;
+      if (tid < 20) reinterpret_cast<double*>(&c->x)[tid] = reinterpret_cast<const double*>(&c->xstart)[tid];
+      return;
+    }
   }
-  if (tid < NS) c->bs[tid] = gyro && held_gyro_only(tid) ? 0.0 : bs[tid];
-  if (tid == 0) {
-    c->x = c->x1;
-    c->xbar = c->x1;
+  if (tid < 20) {
+    const double v = reinterpret_cast<const double*>(&c->x1)[tid];
+    reinterpret_cast<double*>(&c->x)[tid] = v;
+    reinterpret_cast<double*>(&c->xbar)[tid] = v;
+  } else if (tid >= 32 && tid < 41) {
+    c->Rref[tid - 32] = quat_rot_e(c->x1.q, tid - 32);
+  } else if (tid >= 41 && tid < 44) {
+    c->rref[tid - 41] = c->x1.r[tid - 41];
+  } else if (tid == 64) {
     c->t_state = sp.imu->t1;
-    load_pose_ref(c);
     c->ref_index = 1 - c->ref_index;
   }
 }
@@ -1916,11 +2025,11 @@ __global__ void __launch_bounds__(kSolveThreads) k_linearise_end(SolveParams sp,
   }
 }
 
-// Slot blockIdx.x of a batched launch: its SolveParams with this launch's IMU
-// block, level and last-iteration flag, copied to shared memory; returns the
-// slot's mode (uniform over the block).
-__device__ int load_slot_params(const BatchArgs& a, SolveParams& sp) {
-  const int slot = a.slot0 + blockIdx.x;
+// Slot i of a batched launch (blockIdx.x by default): its SolveParams with this
+// launch's IMU block, level and last-iteration flag, copied to shared memory; returns
+// the slot's mode (uniform over the block).
+__device__ int load_slot_params(const BatchArgs& a, SolveParams& sp, int i = -1) {
+  const int slot = a.slot0 + (i < 0 ? blockIdx.x : i);
   const SlotDyn& d = batch_dyn(a, slot);
   // the record and the parameters are loaded in one round; the per-launch fields
   // (imu, level, last) are written by their own thread
@@ -1954,18 +2063,20 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_gn_step_batch(const BatchA
   __shared__ SolveParams sp;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   grid_dep_launch();                    // the next pixel kernel waits for this step itself
-  const int mode = load_slot_params(a, sp);
-  if (mode == kSlotTrack && sp.gdof == 3) {
-    gn_step_g3(sp, *reinterpret_cast<Gn3Smem*>(smem_raw));
-  } else if (mode == kSlotTrack) {
-    // the covariance form, except where the full system is wanted (marginalisation
-    // after the last iteration) or the frame's prior does not allow it
-    if (sp.track_mode == DRI_TRACK_RGBD_ONLY)
-      gn_step_pose_only(sp, *reinterpret_cast<FastSmem*>(smem_raw));
-    else if (sp.last || !gn_step_fast(sp, *reinterpret_cast<FastSmem*>(smem_raw)))
-      gn_step_body(sp, *reinterpret_cast<GnSmem*>(smem_raw));
-  } else {
+  const bool lin = (int)blockIdx.x >= a.nslots;        // a frame's last launch has two blocks per slot
+  const int mode = load_slot_params(a, sp, lin ? blockIdx.x - a.nslots : blockIdx.x);
+  if (mode != kSlotTrack) {
     grid_dep_wait();                    // idle slot: nothing to read, keep the ordering
+  } else if (sp.gdof == 3) {
+    if (!lin) gn_step_g3(sp, *reinterpret_cast<Gn3Smem*>(smem_raw));
+  } else if (sp.track_mode == DRI_TRACK_RGBD_ONLY) {
+    if (!lin) gn_step_pose_only(sp, *reinterpret_cast<FastSmem*>(smem_raw));
+  } else if (lin) {
+    step_lin_block(sp, *reinterpret_cast<GnSmem*>(smem_raw));
+  } else {
+    // the covariance form, except where the frame's prior does not allow it
+    if (!gn_step_fast(sp, *reinterpret_cast<FastSmem*>(smem_raw)))
+      gn_step_body(sp, *reinterpret_cast<GnSmem*>(smem_raw));
   }
 }
 
@@ -1975,9 +2086,11 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_gn_step_batch(const BatchA
 __global__ void __launch_bounds__(kSolveThreads) k_frame_end_batch(const BatchArgs a) {
   __shared__ SolveParams sp;
   const int mode = load_slot_params(a, sp);
+  extern __shared__ __align__(16) unsigned char smem_raw[];
   if (mode == kSlotTrack) {
-    if (sp.gdof == 3) frame_end_body<18>(sp);
-    else frame_end_body<17>(sp);
+    EndSmem& E = *reinterpret_cast<EndSmem*>(smem_raw);
+    if (sp.gdof == 3) frame_end_body<18>(sp, E);
+    else frame_end_body<17>(sp, E);
   } else if (mode == kSlotInit) {
     if (sp.gdof == 3) frame_init_body<18>(sp);
     else frame_init_body<17>(sp);
@@ -2032,7 +2145,7 @@ int launch_priority(bool solver) {
 
 cudaError_t launch_gn_step_batch(const BatchArgs& a, bool g3, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(a.nslots);
+  cfg.gridDim = dim3(a.last ? 2 * a.nslots : a.nslots);
   cfg.blockDim = dim3(kSolveThreads);
   cfg.dynamicSmemBytes = g3 ? kGnSmemMax : kGnSmem2;
   cfg.stream = s;
@@ -2046,7 +2159,7 @@ cudaError_t launch_gn_step_batch(const BatchArgs& a, bool g3, cudaStream_t s) {
   return cudaLaunchKernelEx(&cfg, k_gn_step_batch, a);
 }
 cudaError_t launch_frame_end_batch(const BatchArgs& a, cudaStream_t s) {
-  k_frame_end_batch<<<a.nslots, kSolveThreads, 0, s>>>(a);
+  k_frame_end_batch<<<a.nslots, kSolveThreads, sizeof(EndSmem), s>>>(a);
   return cudaGetLastError();
 }
 cudaError_t launch_gather_heads(const BatchArgs& a, unsigned char* out, cudaStream_t s) {
