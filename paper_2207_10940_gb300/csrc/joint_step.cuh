@@ -1209,79 +1209,107 @@ __device__ void gn_step_pose_only(const SolveParams& sp, FastSmem& S) {
 
 // ---- the frame's constants (k_frame_begin) -----------------------------------------
 
-// Fills Ctrl::elim for the frame: the sweep operator over y (components 6..16) of
-// the prior's augmented matrix [H* b*] leaves -P = -H_yy^-1, P H_yp = -K, P b_y and,
-// on the pose block, the Schur complement and its vector; element-parallel on the
-// lower triangle, one of its 170 entries per thread (per pivot a reciprocal, a
-// scaling and an update).  Components that the gyro-only variant holds are left
-// out (zero rows and columns).  pk, dt: the frame's np pieces; Sg: the 9 x 9
-// covariance of the (r, a, v) rows.  Whole block.  elim.ok stays 0 when H_yy is
-// not safely positive definite or there are more pieces than the step keeps in
-// shared memory: the frame's steps then all take the information form.
+// Reciprocal of a positive pivot to FP64 rounding (two Newton steps): the frame's
+// constants and the marginalisation subtract large terms from one another.
+__device__ __forceinline__ double pivot_recip_full(double d) {
+  const double y = pivot_recip(d);
+  return fma(y, fma(-d, y, 1.0), y);
+}
+
+// Entry (i, j) of a symmetric matrix after the sweep operator on index k: -1 / d on the
+// pivot, a / d in its row and column, a - c_i c_j / d elsewhere; c: column k, r = 1 / d.
+// Swept over an index set Y, the matrix holds -(A_YY)^-1, (A_YY)^-1 A_Y. and the Schur
+// complement.
+__device__ __forceinline__ double sweep_entry(int i, int j, int k, double v, const double* c, double r) {
+  const double t = c[max(i, 0)] * c[max(j, 0)];
+  const bool ik = i == k, jk = j == k;
+  return fma(ik && jk ? -1.0 : ik || jk ? v : -t, r, ik || jk ? 0.0 : v);
+}
+
+// Fills Ctrl::elim for the frame: the sweep operator over y (components 6..16) of the
+// prior's augmented matrix [H* b*] leaves -P = -H_yy^-1, P H_yp = -K, P b_y and, on the
+// pose block, the Schur complement and its vector; element-parallel on its 170 entries,
+// two per thread of warps 0-3.  Components that the gyro-only variant holds are left
+// out (zero rows and columns).  pk, dt: the frame's np pieces; Sg: the 9 x 9 covariance
+// of the (r, a, v) rows.  Warps 0-5 (4 and 5 store the pieces and the covariance
+// blocks).  elim.ok stays 0 when H_yy is not safely positive definite or there are more
+// pieces than the step keeps in shared memory: the frame's steps then all take the
+// information form.
 __device__ void prepare_elim(const SolveParams& sp, Ctrl* c, int np, const double* dt, const int* pk,
-                             double T, const double* Sg, double* col, int* bad) {
+                             double T, const double* Sg, double (*col)[18], double* sink, int* bad) {
   const int tid = threadIdx.x;
-  const bool gyro = sp.track_mode == DRI_TRACK_GYRO_ONLY;
-  int i = -1, j = -1;
-  double v = 0.0;
-  if (tid < 170) {                    // rows 0..16, then the row of b* (17)
-    if (tid < 153) {
-      i = (int)((sqrtf(8.f * tid + 1.f) - 1.f) * 0.5f);
-      while (tri(i + 1, 0) <= tid) ++i;
-      while (tri(i, 0) > tid) --i;
-      j = tid - tri(i, 0);
-      v = c->Hs[i * 17 + j];
-    } else {
-      i = 17;
-      j = tid - 153;
-      v = c->bs[j];
+  double* m = c->elim.m;
+  if (tid >= 128) {
+    const int t = tid - 128;
+    if (np <= kElimPieces) {
+      const dri_imu_sample* s = imu_samples(sp.imu);
+      for (int L = t; L < 8 * np; L += 64) {
+        const int k = L >> 3, q = L & 7;
+        const dri_imu_sample& x = s[pk[k]];
+        c->elim.piece[k][q] = q == 0 ? dt[k] : q == 1 ? 0.5 * dt[k] : q < 5 ? x.gyr[q - 2] : x.acc[q - 5];
+      }
     }
-    if (gyro && ((i < 17 && held_gyro_only(i)) || held_gyro_only(j))) v = 0.0;
+    if (t < 54) {
+      if (t < 36) m[kElS6 + t] = Sg[(t / 6) * 9 + t % 6];
+      else m[kElSv + t - 36] = Sg[(6 + (t - 36) / 6) * 9 + (t - 36) % 6];
+    } else if (t == 54) {
+      m[kElSg] = sp.sigma_grav * sp.sigma_grav;
+      m[kElT] = T;
+    }
+    return;
+  }
+  const bool gyro = sp.track_mode == DRI_TRACK_GYRO_ONLY;
+  int ei[2], ej[2];
+  double v[2], diag[2];
+#pragma unroll
+  for (int o = 0; o < 2; ++o) {
+    const int e = tid + 128 * o;      // rows 0..16, then the row of b* (17)
+    int i = -1, j = -1;
+    double x = 0.0;
+    if (e < 170) {
+      i = e < 153 ? (int)((sqrtf(8.f * e + 1.f) - 1.f) * 0.5f) : 17;
+      if (e < 153 && tri(i + 1, 0) <= e) ++i;
+      if (e < 153 && tri(i, 0) > e) --i;
+      j = e - tri(i, 0);
+      x = i < 17 ? c->Hs[i * 17 + j] : c->bs[j];
+      if (gyro && ((i < 17 && held_gyro_only(i)) || held_gyro_only(j))) x = 0.0;
+    }
+    ei[o] = i;
+    ej[o] = j;
+    v[o] = diag[o] = x;
   }
   if (tid == 0) *bad = np > kElimPieces;
-  const double diag = v;
-  double* m = c->elim.m;
-  if (np <= kElimPieces) {
-    const dri_imu_sample* s = imu_samples(sp.imu);
-    for (int L = tid; L < 8 * np; L += kSolveThreads) {
-      const int k = L >> 3, q = L & 7;
-      const dri_imu_sample& x = s[pk[k]];
-      c->elim.piece[k][q] = q == 0 ? dt[k] : q == 1 ? 0.5 * dt[k] : q < 5 ? x.gyr[q - 2] : x.acc[q - 5];
-    }
-  }
-  for (int e = tid; e < 54; e += kSolveThreads) {
-    if (e < 36) m[kElS6 + e] = Sg[(e / 6) * 9 + e % 6];
-    else m[kElSv + e - 36] = Sg[(6 + (e - 36) / 6) * 9 + (e - 36) % 6];
-  }
-  if (tid == 0) {
-    m[kElSg] = sp.sigma_grav * sp.sigma_grav;
-    m[kElT] = T;
-  }
-  __syncthreads();
+  bar_sync<1, 128>();
+#pragma unroll 1
   for (int k = 6; k < 17; ++k) {
     if (gyro && held_gyro_only(k)) continue;
-    double* ck = col + (k & 1) * 18;  // column k by symmetry
-    if (i == k) ck[j] = v;
-    else if (j == k) ck[i] = v;
-    if (i == k && j == k && !(v > 1e-12 * diag && v < 1e300)) *bad = 1;
-    __syncthreads();
-    const double r = pivot_recip(ck[k]);
-    if (i >= 0) {
-      if (i == k && j == k) v = -r;
-      else if (i == k || j == k) v = v * r;
-      else v = fma(-(ck[i] * r), ck[j], v);
+    double* ck = col[k & 1];          // column k by symmetry
+#pragma unroll
+    for (int o = 0; o < 2; ++o) {
+      const int i = ei[o], j = ej[o];
+      *(i == k ? ck + j : j == k ? ck + i : sink + tid) = v[o];
+      if (i == k && j == k && !(v[o] > 1e-12 * diag[o] && v[o] < 1e29)) *bad = 1;
     }
+    bar_sync<1, 128>();
+    const double r = pivot_recip_full(ck[k]);
+#pragma unroll
+    for (int o = 0; o < 2; ++o) v[o] = sweep_entry(ei[o], ej[o], k, v[o], ck, r);
   }
-  if (i == 17) {
-    m[j < 6 ? kElBp + j : kElM0 + j - 6] = v;
-  } else if (i >= 6 && j >= 6) {
-    m[kElPy + (i - 6) * 11 + j - 6] = -v;
-    m[kElPy + (j - 6) * 11 + i - 6] = -v;
-  } else if (i >= 6) {
-    m[kElK + (i - 6) * 6 + j] = -v;
-  } else if (i >= 0) {
-    m[kElHp + i * 6 + j] = v;
-    m[kElHp + j * 6 + i] = v;
+  bar_sync<1, 128>();
+#pragma unroll
+  for (int o = 0; o < 2; ++o) {
+    const int i = ei[o], j = ej[o];
+    if (i == 17) {
+      m[j < 6 ? kElBp + j : kElM0 + j - 6] = v[o];
+    } else if (i >= 6 && j >= 6) {
+      m[kElPy + (i - 6) * 11 + j - 6] = -v[o];
+      m[kElPy + (j - 6) * 11 + i - 6] = -v[o];
+    } else if (i >= 6) {
+      m[kElK + (i - 6) * 6 + j] = -v[o];
+    } else if (i >= 0) {
+      m[kElHp + i * 6 + j] = v[o];
+      m[kElHp + j * 6 + i] = v[o];
+    }
   }
   if (tid == 0) {
     c->elim.np = np;

@@ -121,31 +121,26 @@ struct ImuWork {
   int np;
 };
 
-// Row r (0..8, order phi, v, p) of piece k's gyro-noise gain to the end of the
-// interval, divided by dt_k.
-__device__ __forceinline__ void gyro_gain_row(const ImuWork& W, int np, int k, int r, double* o) {
-  const double* Yp = W.Y[k];
+// Element (r, m) (row r of 0..8, order phi, v, p) of piece k's gyro-noise gain to the
+// end of the interval, divided by dt_k.
+__device__ __forceinline__ double gyro_gain_e(const ImuWork& W, int np, int k, int r, int m) {
+  const double* Yp = W.Y[k] + m;
+  const int rr = r % 3;
   if (r < 3) {
-    const double* R = W.dR[np];
-#pragma unroll
-    for (int m = 0; m < 3; ++m) o[m] = R[r] * Yp[m] + R[3 + r] * Yp[3 + m] + R[6 + r] * Yp[6 + m];
-  } else {
-    const double* v = (r < 6 ? W.Cv : W.Dv)[k + 1];
-    const int rr = r % 3;
-    double h0, h1, h2;   // row rr of [v]x
-    if (rr == 0) { h0 = 0.0; h1 = -v[2]; h2 = v[1]; }
-    else if (rr == 1) { h0 = v[2]; h1 = 0.0; h2 = -v[0]; }
-    else { h0 = -v[1]; h1 = v[0]; h2 = 0.0; }
-#pragma unroll
-    for (int m = 0; m < 3; ++m) o[m] = -(h0 * Yp[m] + h1 * Yp[3 + m] + h2 * Yp[6 + m]);
+    const double* R = W.dR[np] + rr;
+    return fma(R[0], Yp[0], fma(R[3], Yp[3], R[6] * Yp[6]));
   }
+  const double* v = (r < 6 ? W.Cv : W.Dv)[k + 1];
+  const int r1 = rr == 2 ? 0 : rr + 1, r2 = rr == 0 ? 2 : rr - 1;
+  return fma(v[r2], Yp[3 * r1], -(v[r1] * Yp[3 * r2]));       // -(v x column m)_rr
 }
 
 // Whole block.  Pre-integration at biases (bg, ba) into P (and the noise
-// covariance when cov).  Returns false (for all threads) if the samples do not
+// covariance when cov, through gain, kMaxPieces x 27 scratch).  Returns false (for all threads) if the samples do not
 // cover the interval.
 __device__ bool preintegrate_block(const ImuHeader* h, const double* bg, const double* ba, bool cov,
-                                   double gnd, double and_, ImuWork& W, Preint& P) {
+                                   double gnd, double and_, ImuWork& W, Preint& P,
+                                   double (*gain)[27] = nullptr) {
   const int tid = threadIdx.x, nt = blockDim.x;
   const int warp = tid >> 5, lane = tid & 31;
   const dri_imu_sample* s = imu_samples(h);
@@ -296,12 +291,22 @@ __device__ bool preintegrate_block(const ImuHeader* h, const double* bg, const d
     }
   }
   __syncthreads();
-  if (warp == 0 && lane < 6) {         // dv, dp
+  // the sums over the pieces run on four warps, the covariance (which has 45 of them)
+  // on three others
+  const int sw = cov ? warp - 4 : warp;
+  if (cov) {
+    for (int L = tid; L < 27 * np; L += nt) {
+      const int k = L / 27, e = L - 27 * k;
+      gain[k][e] = gyro_gain_e(W, np, k, e / 3, e % 3);
+    }
+    __syncthreads();
+  }
+  if (sw == 0 && lane < 6) {           // dv, dp
     const int i = lane % 3;
     double acc = 0.0;
     for (int k = 0; k < np; ++k) acc += W.u[k][i] * (lane < 3 ? W.dt[k] : W.w[k]);
     (lane < 3 ? P.dv : P.dp)[i] = acc;
-  } else if (warp == 1 && lane < 18) { // d(dv, dp)/d(b_g) = -sum [u_k]x Psi_k (dt_k | w_k)
+  } else if (sw == 3 && lane < 18) {   // d(dv, dp)/d(b_g) = -sum [u_k]x Psi_k (dt_k | w_k)
     const int e = lane % 9, r = e / 3, c = e % 3, r1 = (r + 1) % 3, r2 = (r + 2) % 3;
     double acc = 0.0;
     for (int k = 0; k < np; ++k) {
@@ -311,38 +316,38 @@ __device__ bool preintegrate_block(const ImuHeader* h, const double* bg, const d
       acc -= hv * (lane < 9 ? W.dt[k] : W.w[k]);
     }
     (lane < 9 ? P.Vg : P.Pg)[e] = acc;
-  } else if (warp == 2 && lane < 18) { // d(dv, dp)/d(b_a) = -sum dR_k (dt_k | w_k)
+  } else if (sw == 1 && lane < 18) {   // d(dv, dp)/d(b_a) = -sum dR_k (dt_k | w_k)
     const int e = lane % 9;
     double acc = 0.0;
     for (int k = 0; k < np; ++k) acc -= W.dR[k][e] * (lane < 9 ? W.dt[k] : W.w[k]);
     (lane < 9 ? P.Va : P.Pa)[e] = acc;
-  } else if (warp == 3 && lane < 9) {  // d(dR)/d(b_g) = dR_N^T Psi_N
+  } else if (sw == 2 && lane < 9) {    // d(dR)/d(b_g) = dR_N^T Psi_N
     const int r = lane / 3, c = lane % 3;
     const double* R = W.dR[np];
     const double* Ps = W.EP[np];
     P.Phig[lane] = R[r] * Ps[c] + R[3 + r] * Ps[3 + c] + R[6 + r] * Ps[6 + c];
     P.dR[lane] = R[lane];
-  } else if (cov && tid >= 128 && tid < 128 + 45) {
-    // covariance entry (r, c), r <= c, of (dphi, dv, dp)
-    int e = tid - 128, r = 0;
+  } else if (cov && tid < 96) {
+    // covariance entry (r, c), r <= c, of (dphi, dv, dp): two lanes per entry, every
+    // second piece each (one lane for all pieces, forming the gains itself: 60k cycles
+    // of the frame start's 152k)
+    int e = min(tid >> 1, 44), r = 0;
     while (e >= 9 - r) { e -= 9 - r; ++r; }
     const int c = r + e;
-    double acc = 0.0;
-    const double q_g = gnd * gnd, q_a = and_ * and_;
-    for (int k = 0; k < np; ++k) {
+    double sg = 0.0, sa = 0.0;
+    for (int k = tid & 1; k < np; k += 2) {
       const double dt = W.dt[k];
-      double gr[3], gc[3];
-      gyro_gain_row(W, np, k, r, gr);
-      gyro_gain_row(W, np, k, c, gc);
-      acc += q_g * dt * (gr[0] * gc[0] + gr[1] * gc[1] + gr[2] * gc[2]);
-      if (r >= 3 && (r % 3) == (c % 3)) {   // accelerometer noise: v and p blocks
-        const double ck = (T - W.tau[k + 1]) + 0.5 * dt;
-        const double fr = r < 6 ? 1.0 : ck, fc = c < 6 ? 1.0 : ck;
-        acc += q_a * dt * fr * fc;
-      }
+      const double* gr = gain[k] + 3 * r;
+      const double* gc = gain[k] + 3 * c;
+      sg = fma(dt, fma(gr[0], gc[0], fma(gr[1], gc[1], gr[2] * gc[2])), sg);
+      const double ck = fma(0.5, dt, T - W.tau[k + 1]);       // accelerometer noise: v and p blocks
+      sa = fma(dt, (r < 6 ? 1.0 : ck) * (c < 6 ? 1.0 : ck), sa);
     }
-    P.Sig[r * 9 + c] = acc;
-    P.Sig[c * 9 + r] = acc;
+    sg += __shfl_xor_sync(0xffffffffu, sg, 1);
+    sa += __shfl_xor_sync(0xffffffffu, sa, 1);
+    const double v = gnd * gnd * sg + (r >= 3 && (r % 3) == (c % 3) ? and_ * and_ * sa : 0.0);
+    P.Sig[r * 9 + c] = v;
+    P.Sig[c * 9 + r] = v;
   }
   if (tid == 0) P.T = T;
   __syncthreads();
@@ -701,48 +706,6 @@ __device__ void warp_write_transforms(Ctrl* c, const DState& x0, const DState& x
 // ---------------------------------------------------------------------------
 // dense symmetric factorisation
 // ---------------------------------------------------------------------------
-
-// In-place LDL^T of the symmetric n x n matrix in A (lower triangle read): the
-// strict lower triangle becomes the unit-lower L, the diagonal D.  Whole block;
-// col is shared scratch of 2 n doubles, fail a shared int.  False (for all
-// threads) if a pivot is not positive.
-__device__ bool block_ldlt(double* A, int n, int ld, double* col, int* fail) {
-  const int tid = threadIdx.x, nt = blockDim.x;
-  if (tid == 0) *fail = 0;
-  __syncthreads();
-  for (int k = 0; k < n; ++k) {
-    const double d = A[k * ld + k];
-    if (tid == 0 && !(d > 0.0 && d < INFINITY)) *fail = 1;
-    double* ck = col + (k & 1) * n;
-    const double* cp = col + ((k + 1) & 1) * n;
-    for (int i = k + 1 + tid; i < n; i += nt) ck[i] = A[i * ld + k] / d;
-    if (k > 0)
-      for (int i = k + tid; i < n; i += nt) A[i * ld + (k - 1)] = cp[i];
-    __syncthreads();
-    const int m = n - k - 1;
-    for (int p = tid; p < m * m; p += nt) {
-      const int i = k + 1 + p / m, j = k + 1 + p % m;
-      if (j <= i) A[i * ld + j] -= A[i * ld + k] * ck[j];
-    }
-    __syncthreads();
-  }
-  return *fail == 0;
-}
-
-// The same for one right-hand side in one thread.
-__device__ void ldlt_solve_thread(const double* A, int n, int ld, double* b) {
-  for (int i = 0; i < n; ++i) {
-    double s = b[i];
-    for (int k = 0; k < i; ++k) s -= A[i * ld + k] * b[k];
-    b[i] = s;
-  }
-  for (int i = 0; i < n; ++i) b[i] /= A[i * ld + i];
-  for (int i = n - 1; i >= 0; --i) {
-    double s = b[i];
-    for (int k = i + 1; k < n; ++k) s -= A[k * ld + i] * b[k];
-    b[i] = s;
-  }
-}
 
 // Pivot reciprocal: an FP32 seed refined by one Newton-Raphson step (relative
 // error below 2^-44.8; the factorisation is then exact for a matrix whose pivots
@@ -1610,11 +1573,14 @@ struct BeginSmem {
   ImuWork W;
   Preint P;
   ImuLin L;
+  double gain[kMaxPieces][27];
   double G[81], GS[81], Sg[81], Winv[81];
-  double col[18];
-  double ecol[36];
+  double col[2][10];
+  double ecol[2][18], sink[128];
   double rot[18];
-  int ok, fail;
+  DState x1;
+  double dx[17];
+  int ok, fail, elim_bad;
 };
 
 __device__ bool imu_weight_and_prediction(const SolveParams& sp, Ctrl* c, BeginSmem& B,
@@ -1627,7 +1593,7 @@ __device__ bool imu_weight_and_prediction(const SolveParams& sp, Ctrl* c, BeginS
   __syncthreads();
   if (!B.ok) return false;
   const DState x0 = c->x0;
-  if (!preintegrate_block(sp.imu, x0.bg, x0.ba, true, sp.gyr_nd, sp.acc_nd, B.W, B.P)) {
+  if (!preintegrate_block(sp.imu, x0.bg, x0.ba, true, sp.gyr_nd, sp.acc_nd, B.W, B.P, B.gain)) {
     if (tid == 0) c->status = DRI_ENOTREADY;
     return false;
   }
@@ -1680,43 +1646,73 @@ __device__ bool imu_weight_and_prediction(const SolveParams& sp, Ctrl* c, BeginS
   __syncthreads();
   if (tid < 81) B.Sg[tid] = sym;
   __syncthreads();
-  if (sp.gdof != 3) {                 // the steps' constants (joint_step.cuh)
-    prepare_elim(sp, c, B.W.np, B.W.dt, B.W.pk, B.P.T, B.Sg, B.ecol, &B.fail);
-    __syncthreads();
-  }
-  const bool pd = block_ldlt(B.Sg, 9, 9, B.col, &B.fail);
-  if (tid < 9) {
-    double colv[9];
-    for (int i = 0; i < 9; ++i) colv[i] = (i == tid) ? 1.0 : 0.0;
-    ldlt_solve_thread(B.Sg, 9, 9, colv);
-    for (int i = 0; i < 9; ++i) B.Winv[i * 9 + tid] = colv[i];
+  // side by side: the steps' constants (warps 0-5; joint_step.cuh) and Sigma^-1
+  // (warps 6-7: a sweep of its 45 entries, one per thread)
+  const int warp = tid >> 5, lane = tid & 31;
+  if (warp < 6) {
+    if (sp.gdof != 3) prepare_elim(sp, c, B.W.np, B.W.dt, B.W.pk, B.P.T, B.Sg, B.ecol, B.sink, &B.elim_bad);
+  } else {
+    const int t = tid - 192;
+    int i = -1, j = -1;
+    if (t < 45) {
+      i = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
+      if (tri(i + 1, 0) <= t) ++i;
+      if (tri(i, 0) > t) --i;
+      j = t - tri(i, 0);
+    }
+    double v = i < 0 ? 0.0 : B.Sg[i * 9 + j];
+    bool good = true;
+#pragma unroll 1
+    for (int k = 0; k < 9; ++k) {
+      double* ck = B.col[k & 1];
+      if (i == k) ck[j] = v;
+      else if (j == k) ck[i] = v;
+      bar_sync<2, 64>();
+      const double d = ck[k];
+      good = good && __double2hiint(d) > 0 && finite_bits(d);
+      v = sweep_entry(i, j, k, v, ck, pivot_recip_full(d));
+    }
+    if (i >= 0) B.Winv[i * 9 + j] = B.Winv[j * 9 + i] = -v;
+    if (t == 0) B.fail = !good;
   }
   __syncthreads();
-  for (int idx = tid; idx < 18 * 18; idx += blockDim.x) {
-    const int r = idx / 18, q = idx % 18;
-    double w = 0.0;
-    if (r < 9 && q < 9) {
-      if (!gyro || (r >= 3 && r < 6 && q >= 3 && q < 6)) w = 0.5 * (B.Winv[r * 9 + q] + B.Winv[q * 9 + r]);
-    } else if (r == q) {
-      if (r < 12) w = 1.0 / (sp.gyr_rw * sp.gyr_rw * B.P.T);
-      else if (gyro) w = 0.0;                  // accelerometer bias and gravity rows
-      else if (r < 15) w = 1.0 / (sp.acc_rw * sp.acc_rw * B.P.T);
-      else w = 1.0 / (sp.sigma_grav * sp.sigma_grav);
+  const bool pd = !B.fail;
+  if (warp > 0) {
+    for (int idx = tid - 32; idx < 18 * 18; idx += kSolveThreads - 32) {
+      const int r = idx / 18, q = idx % 18;
+      double w = 0.0;
+      if (r < 9 && q < 9) {
+        if (!gyro || (r >= 3 && r < 6 && q >= 3 && q < 6)) w = B.Winv[r * 9 + q];
+      } else if (r == q) {
+        if (r < 12) w = 1.0 / (sp.gyr_rw * sp.gyr_rw * B.P.T);
+        else if (gyro) w = 0.0;                  // accelerometer bias and gravity rows
+        else if (r < 15) w = 1.0 / (sp.acc_rw * sp.acc_rw * B.P.T);
+        else w = 1.0 / (sp.sigma_grav * sp.sigma_grav);
+      }
+      c->Wimu[idx] = w;
     }
-    c->Wimu[idx] = w;
-  }
-  if (tid == 0) {
-    if (!pd) c->status = DRI_ELOST;
+  } else {
+    if (lane == 0 && !pd) c->status = DRI_ELOST;
     if (x1_pred) {
       // x1 := x^1(x0): biases and q_IW carried over; gyro only: the predicted
-      // rotation at x0's position and velocity
-      DState x1 = x0;
-      for (int i = 0; i < 3 && !gyro; ++i) {
-        x1.r[i] = B.L.r[i];
-        x1.v[i] = B.L.v[i];
+      // rotation at x0's position and velocity.  The quaternion is exp(log(R^)).
+      if (lane < 17) B.dx[lane] = 0.0;
+      if (lane < 20) reinterpret_cast<double*>(&B.x1)[lane] = reinterpret_cast<const double*>(&c->x0)[lane];
+      __syncwarp();
+      if (lane < 3) {
+        B.dx[3 + lane] = log_i(B.L.Rh, lane);
+        if (!gyro) {
+          B.x1.r[lane] = B.L.r[lane];
+          B.x1.v[lane] = B.L.v[lane];
+        }
       }
-      rot_to_quat(B.L.Rh, x1.q);
-      *x1_pred = x1;
+      if (lane < 4) B.x1.q[lane] = lane == 0 ? 1.0 : 0.0;
+      __syncwarp();
+      const double qg = lane < 4 ? B.x1.qg[lane] : 0.0;
+      fast_boxplus(B.x1, B.dx);
+      if (lane < 4) B.x1.qg[lane] = qg;          // carried over as it is
+      __syncwarp();
+      if (lane < 20) reinterpret_cast<double*>(x1_pred)[lane] = reinterpret_cast<const double*>(&B.x1)[lane];
     }
   }
   __syncthreads();
@@ -1779,13 +1775,6 @@ struct EndSmem : PixSmem {
   double R0[9], Rref[9], dr[3];
   int ok, bad;
 };
-
-// Reciprocal of a positive pivot to FP64 rounding (two Newton steps): the
-// marginalisation subtracts large terms (the IMU weights) from one another.
-__device__ __forceinline__ double pivot_recip_full(double d) {
-  const double y = pivot_recip(d);
-  return fma(y, fma(-d, y, 1.0), y);
-}
 
 // Schur complement (Eq. 8) of the leading NS x NS block of [H | bp] (row-major 2 NS,
 // full) onto the trailing one: element-parallel elimination on warps 0-3, an entry of
