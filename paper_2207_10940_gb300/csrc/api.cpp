@@ -606,6 +606,7 @@ BatchArgs plan_args(const Plan* p, size_t start_off, int level, int last, int sl
   a.nslots = nslots < 0 ? p->S : nslots;
   a.level = level;
   a.last = last;
+  for (int i = 0; a.nslots <= kArgCtrls && i < a.nslots; ++i) a.ctrl[i] = p->slots[slot0 + i]->ctrl;
   return a;
 }
 

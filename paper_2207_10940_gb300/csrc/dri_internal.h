@@ -211,6 +211,8 @@ struct TableView {
 };
 TableView table_view(int nslots, int levels, int groups);
 
+constexpr int kArgCtrls = 16;
+
 // Kernel argument of every batched launch: it covers slots slot0 ..
 // slot0 + nslots - 1 of the plan (all of them, or one group of the
 // Gauss-Newton loop).
@@ -218,6 +220,7 @@ struct BatchArgs {
   const SlotStatic* slots;            // every slot of the plan
   const unsigned char* dyn;           // SlotDyn[all slots], then the IMU blocks
   const int32_t* start;               // block prefix over this launch's slots (nslots + 1)
+  Ctrl* ctrl[kArgCtrls];                     // the slots' control blocks, when nslots <= kArgCtrls
   int32_t slot0;
   int32_t nslots;
   int32_t level;

@@ -95,7 +95,7 @@ struct FastSmem : PixSmem {
   double rot[24];
   double fo[21];
   double cost;
-  int good[2], posdef[4];
+  int good, posdef[4];
 };
 template <int N>
 struct Slots {
@@ -582,14 +582,17 @@ __device__ void fast_pixel_terms(const SolveParams& sp, const Ctrl* c, PixSmem& 
 
 // ---- the sweep ---------------------------------------------------------------------
 
-// x <- x boxplus d by one warp, as warp_state_boxplus: the series of a quaternion
-// group's four components run on its four lanes (cosine on the first, sine on the
-// others), cut where the next term is below 1e-17 for small steps.
-__device__ __forceinline__ void fast_boxplus(DState& x, const double* d) {
+// q <- exp(d) (x) q of two quaternions by one warp, as in warp_state_boxplus: (q0, d0) on
+// lanes 0-3 and (q1, d1) on lanes 4-7 (flat: the third component of d taken as zero).
+// The series of a quaternion's four components run on its four lanes (cosine on the
+// first, sine on the others), cut where the next term is below 1e-17 for small steps.
+__device__ __forceinline__ void fast_quat_boxplus(double* q0, const double* d0, bool flat0, double* q1,
+                                                  const double* d1, bool flat1) {
   const int lane = threadIdx.x & 31, grp = (lane >> 2) & 1, k = lane & 3, base = lane & ~3;
-  double* q = grp ? x.qg : x.q;
-  const double d0 = grp ? d[15] : d[3], d1 = grp ? d[16] : d[4], d2 = grp ? 0.0 : d[5];
-  const double t2 = fma(d0, d0, fma(d1, d1, d2 * d2));
+  double* q = grp ? q1 : q0;
+  const double* d = grp ? d1 : d0;
+  const double dx = d[0], dy = d[1], dz = (grp ? flat1 : flat0) ? 0.0 : d[2];
+  const double t2 = fma(dx, dx, fma(dy, dy, dz * dz));
   double f;
   if (__all_sync(0xffffffffu, pos_less(t2, 1e-6))) {
     f = fma(t2, fma(t2, k ? 1.0 / 3840 : 1.0 / 384, k ? -1.0 / 48 : -1.0 / 8), k ? 0.5 : 1.0);
@@ -603,7 +606,7 @@ __device__ __forceinline__ void fast_boxplus(DState& x, const double* d) {
     sincos(0.5 * t, &sn, &cs);
     f = k ? (t2 > 0.0 ? sn / t : 0.5) : cs;
   }
-  f *= k == 0 ? 1.0 : k == 1 ? d0 : k == 2 ? d1 : d2;
+  f *= k == 0 ? 1.0 : k == 1 ? dx : k == 2 ? dy : dz;
   double o = 0.0;
 #pragma unroll
   for (int j = 0; j < 4; ++j) {      // component k of exp(d) (x) q, as quat_mul_k
@@ -617,6 +620,13 @@ __device__ __forceinline__ void fast_boxplus(DState& x, const double* d) {
   else o *= rsqrt(n2);
   __syncwarp();
   if (lane < 8) q[k] = o;
+  __syncwarp();
+}
+
+// x <- x boxplus d by one warp, as warp_state_boxplus.
+__device__ __forceinline__ void fast_boxplus(DState& x, const double* d) {
+  const int lane = threadIdx.x & 31;
+  fast_quat_boxplus(x.q, d + 3, false, x.qg, d + 15, true);
   if (lane < 12) {
     const int g = lane / 3, i = lane - 3 * g;
     double* v = g == 0 ? x.r : g == 1 ? x.v : g == 2 ? x.bg : x.ba;
@@ -625,7 +635,7 @@ __device__ __forceinline__ void fast_boxplus(DState& x, const double* d) {
   __syncwarp();
 }
 
-// The pixel kernel's transforms, as warp_write_transforms, from shared memory; warp 0.
+// The pixel kernel's transforms, as warp_write_transforms, from shared memory; one warp.
 __device__ __forceinline__ void fast_transforms(Ctrl* c, FastSmem& S) {
   const int lane = threadIdx.x & 31, f = lane / 9, e = lane - 9 * f, r = e / 3, cc = e - 3 * r;
   if (lane < 24) {                    // R1, R0 (2 (v_r v_c + w^2 or +- w v_k) - I); r1 - r_ref, r1 - r0
@@ -650,45 +660,52 @@ __device__ __forceinline__ void fast_transforms(Ctrl* c, FastSmem& S) {
   }
 }
 
-// One Gauss-Newton step; false (for every thread, nothing done) when the frame's
-// constants do not allow this form.  Whole block.
-__device__ bool gn_step_fast(const SolveParams& sp, FastSmem& S) {
+// The step's loads from the control block, issued before anything else (the block's
+// pointer comes with the launch's arguments): status, whether the frame's constants
+// allow the covariance form, and the number of IMU pieces in registers, the rest to
+// shared memory.
+struct FastLoad {
+  int status, usable, np;
+};
+__device__ __forceinline__ FastLoad fast_load(const Ctrl* c, FastSmem& S) {
+  const int tid = threadIdx.x;
+  const FastLoad r = {c->status, c->elim.ok, c->elim.np};
+  const double* e = c->elim.m;
+  const double* p = &c->elim.piece[0][0];
+  double* q = &S.piece[0][0];
+  double v[4];
+  v[0] = p[tid];
+  v[1] = p[tid + kSolveThreads];
+  v[2] = e[tid];
+  v[3] = 0.0;
+  static_assert(kElimPieces * 8 == 2 * kSolveThreads && kElimDoubles - kSolveThreads == 40, "load layout");
+  const double* src = tid < 20 ? reinterpret_cast<const double*>(&c->x0) + tid
+                      : tid < 40 ? reinterpret_cast<const double*>(&c->x1) + tid - 20
+                      : tid < 60 ? reinterpret_cast<const double*>(&c->xbar) + tid - 40
+                      : tid < 69 ? c->Rref + tid - 60
+                      : tid < 109 ? e + kSolveThreads + tid - 69
+                      : tid < 112 ? c->rref + tid - 109 : nullptr;
+  double* dst = tid < 20 ? reinterpret_cast<double*>(&S.x0) + tid
+                : tid < 40 ? reinterpret_cast<double*>(&S.x1) + tid - 20
+                : tid < 60 ? reinterpret_cast<double*>(&S.xbar) + tid - 40
+                : tid < 69 ? S.Rref + tid - 60
+                : tid < 109 ? S.el + kSolveThreads + tid - 69 : S.rref + tid - 109;
+  if (src) v[3] = *src;
+  q[tid] = v[0];
+  q[tid + kSolveThreads] = v[1];
+  S.el[tid] = v[2];
+  if (src) *dst = v[3];
+  return r;
+}
+
+// One Gauss-Newton step on what fast_load brought; false (for every thread, nothing
+// done) when the frame's constants do not allow this form.  Whole block.
+__device__ bool gn_step_fast(const SolveParams& sp, FastSmem& S, Ctrl* c, const FastLoad& fl) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const bool gyro = sp.track_mode == DRI_TRACK_GYRO_ONLY;
-  Ctrl* c = sp.ctrl;
-  const int status = c->status, usable = c->elim.ok, np = c->elim.np;
-  {                                   // everything in one round of independent loads
-    const double* e = c->elim.m;
-    const double* p = &c->elim.piece[0][0];
-    double* q = &S.piece[0][0];
-    double v[4];
-    v[0] = p[tid];
-    v[1] = p[tid + kSolveThreads];
-    v[2] = e[tid];
-    v[3] = 0.0;
-    static_assert(kElimPieces * 8 == 2 * kSolveThreads && kElimDoubles - kSolveThreads == 40, "load layout");
-    const double* src = tid < 20 ? reinterpret_cast<const double*>(&c->x0) + tid
-                        : tid < 40 ? reinterpret_cast<const double*>(&c->x1) + tid - 20
-                        : tid < 60 ? reinterpret_cast<const double*>(&c->xbar) + tid - 40
-                        : tid < 69 ? c->Rref + tid - 60
-                        : tid < 109 ? e + kSolveThreads + tid - 69
-                        : tid < 112 ? c->rref + tid - 109 : nullptr;
-    double* dst = tid < 20 ? reinterpret_cast<double*>(&S.x0) + tid
-                  : tid < 40 ? reinterpret_cast<double*>(&S.x1) + tid - 20
-                  : tid < 60 ? reinterpret_cast<double*>(&S.xbar) + tid - 40
-                  : tid < 69 ? S.Rref + tid - 60
-                  : tid < 109 ? S.el + kSolveThreads + tid - 69 : S.rref + tid - 109;
-    if (src) v[3] = *src;
-    q[tid] = v[0];
-    q[tid + kSolveThreads] = v[1];
-    S.el[tid] = v[2];
-    if (src) *dst = v[3];
-  }
-  if (status != 0) return true;
-  if (!usable) {
-    __syncthreads();                  // the other form reuses this shared memory
-    return false;
-  }
+  const int np = fl.np;
+  if (fl.status != 0) return true;
+  if (!fl.usable) return false;
   // the sweep's entries of this thread (see there): entry e of the lower triangle
   // and the right-hand side row, longest-updated first, and where its value comes
   // from: sign (*p + *q)
@@ -994,52 +1011,53 @@ __device__ bool gn_step_fast(const SolveParams& sp, FastSmem& S) {
     posdef = __all_sync(0xffffffffu, posdef);
     if (lane == 0) S.posdef[warp] = posdef;
     bar_sync<1, 128>();
-    if (warp < 2) {
-      double* dx = S.dx;
-      if (warp == 0) {
-        const double* Lr = S.L[min(lane, kSys - 1)];
-        double y = Lr[kSys], l = Lr[kSys - 1];
+    // The poses are known after 12 of the 19 substitutions: warp 1 moves them and writes
+    // the next pixel kernel's transforms while warp 0 goes on to the other unknowns.
+    double* dx = S.dx;
+    if (warp == 0) {
+      const double* Lr = S.L[min(lane, kSys - 1)];
+      double y = Lr[kSys], l = Lr[kSys - 1];
+      auto substitute = [&](int from, int to) {
 #pragma unroll 1
-        for (int k = kSys - 1; k > 0; --k) {                  // the next column's entry loads a step ahead
+        for (int k = from; k > to; --k) {                     // the next column's entry loads a step ahead
           const double ln = Lr[k - 1];
           y = fma(lane < k ? -l : 0.0, __shfl_sync(0xffffffffu, y, k), y);
           l = ln;
         }
-        if (lane < kSys) S.z[lane] = y;
-        if (lane >= kLam && lane < kSys) dx[lane < kLam + 6 ? lane - kLam : 4 + lane] = y;   // p0 at 0..5, p1 at 17..22
-        bool ok = S.posdef[0] && S.posdef[1] && S.posdef[2] && S.posdef[3];
-        __syncwarp();
-        // y (lanes 0-10: K p0 + m, 16-26: -T^T lambda), dv1's part without y
-        // (11-13: e_v + B9 da0, 27-29: -S_v6 lambda)
-        const double* lam = S.z;
-        const double* p0 = S.z + kLam;
-        const int h = lane & 15;
-        const bool top = lane >= 16;
-        double w = 0.0;
-        if (h < 14) {
-          const double* A = h < 11 ? (top ? &S.T[0][h] : K + 6 * h) : (top ? S.el + kElSv + 6 * (h - 11) : S.B9 + 3 * (h - 11));
-          const int sa = h < 11 && top ? 11 : 1;
-          const double* B = top ? lam : (h < 11 ? p0 : p0 + 3);
-          const int n = h < 11 ? (top ? 7 : 6) : (top ? 6 : 3);
-          w = top ? 0.0 : h < 11 ? S.m[h] : S.ev[h - 11];
-#pragma unroll
-          for (int k = 0; k < 7; ++k)
-            if (k < n) w = fma(top ? -A[k * sa] : A[k * sa], B[k], w);
-        }
-        w += __shfl_down_sync(0xffffffffu, w, 16);
-        if (lane < 11) dx[6 + lane] = w;
-        else if (lane < 14) S.u[lane - 11] = w;            // dv1's part
-        __syncwarp();
-        bool fin = true;
-        if (lane < 17) fin = finite_bits(dx[lane]);
-        ok = __all_sync(0xffffffffu, fin) && ok;
-        if (lane == 0) S.good[0] = ok;
+      };
+      substitute(kSys - 1, kLam);
+      if (lane >= kLam && lane < kSys) {
+        S.z[lane] = y;
+        dx[lane < kLam + 6 ? lane - kLam : 4 + lane] = y;     // p0 at 0..5, p1 at 17..22
       }
-      bar_sync<6, 64>();
-      if (warp == 0) {
-        fast_boxplus(S.x0, dx);
-      } else {
-        const double* y = dx + 6;     // v, b_g, b_a, gravity
+      __syncwarp();
+      bar_arrive<6, 64>();
+      substitute(kLam, 0);
+      if (lane < kLam) S.z[lane] = y;
+      __syncwarp();
+      // y (lanes 0-10: K p0 + m, 16-26: -T^T lambda), dv1's part without y
+      // (11-13: e_v + B9 da0, 27-29: -S_v6 lambda)
+      const double* lam = S.z;
+      const double* p0 = S.z + kLam;
+      const int h = lane & 15;
+      const bool top = lane >= 16;
+      double w = 0.0;
+      if (h < 14) {
+        const double* A = h < 11 ? (top ? &S.T[0][h] : K + 6 * h) : (top ? S.el + kElSv + 6 * (h - 11) : S.B9 + 3 * (h - 11));
+        const int sa = h < 11 && top ? 11 : 1;
+        const double* B = top ? lam : (h < 11 ? p0 : p0 + 3);
+        const int n = h < 11 ? (top ? 7 : 6) : (top ? 6 : 3);
+        w = top ? 0.0 : h < 11 ? S.m[h] : S.ev[h - 11];
+#pragma unroll
+        for (int k = 0; k < 7; ++k)
+          if (k < n) w = fma(top ? -A[k * sa] : A[k * sa], B[k], w);
+      }
+      w += __shfl_down_sync(0xffffffffu, w, 16);
+      if (lane < 11) dx[6 + lane] = w;
+      else if (lane < 14) S.u[lane - 11] = w;                 // dv1's part
+      __syncwarp();
+      {
+        const double* yv = dx + 6;    // v, b_g, b_a, gravity
         // lanes 0-8: dv1, row lane % 3, part lane / 3; 9-14: x1's biases follow x0's;
         // 15-17: e_g + A dg0
         const int i = lane % 3, q = lane / 3;
@@ -1048,18 +1066,18 @@ __device__ bool gn_step_fast(const SolveParams& sp, FastSmem& S) {
         double base = 0.0;
         if (lane < 9) {
           A = q == 0 ? S.B14 + 3 * i : q == 1 ? S.B17 + 3 * i : S.B20 + 2 * i;
-          B = q == 0 ? y + 3 : q == 1 ? y + 6 : y + 9;
+          B = q == 0 ? yv + 3 : q == 1 ? yv + 6 : yv + 9;
           A2 = q == 2 ? &S.one : A + 2;
-          B2 = q == 2 ? y + i : B + 2;
+          B2 = q == 2 ? yv + i : B + 2;
           base = q == 2 ? S.u[i] : 0.0;
           sa = sb = 1;
         } else if (lane < 15) {
           A2 = &S.one;
-          B2 = y + 3 + lane - 9;
+          B2 = yv + 3 + lane - 9;
           base = S.eb[lane - 9];
         } else if (lane < 18) {
           A = S.Ag + 2 * i;
-          B = y + 9;
+          B = yv + 9;
           base = S.eg[i];
           sa = sb = 1;
         }
@@ -1074,23 +1092,31 @@ __device__ bool gn_step_fast(const SolveParams& sp, FastSmem& S) {
           const double* G = S.Gm + 3 * (lane - 18);
           dx[32 + lane - 18] = -fma(G[0], u0, fma(G[1], u1, G[2] * u2));
         }
-        __syncwarp();
-        bool fin = true;
-        if (lane < 17) fin = finite_bits(dx[17 + lane]);
-        fin = __all_sync(0xffffffffu, fin);
-        if (lane == 0) S.good[1] = fin;
-        fast_boxplus(S.x1, dx + 17);
       }
+      __syncwarp();
+      const bool fin = finite_bits(dx[lane]) && finite_bits(dx[32 + (lane & 1)]);
+      const bool ok = __all_sync(0xffffffffu, fin) && S.posdef[0] && S.posdef[1] && S.posdef[2] && S.posdef[3];
+      if (lane == 0) S.good = ok;
+      fast_quat_boxplus(S.x0.qg, dx + 15, true, S.x1.qg, dx + 32, true);
+      if (lane < 18) {                // velocities and biases
+        const int q = lane / 9, i = lane - 9 * q, f = i / 3;
+        DState& x = q ? S.x1 : S.x0;
+        (f == 0 ? x.v : f == 1 ? x.bg : x.ba)[i - 3 * f] += dx[17 * q + 6 + i];
+      }
+    } else if (warp == 1) {
+      bar_sync<6, 64>();
+      fast_quat_boxplus(S.x0.q, dx + 3, false, S.x1.q, dx + 20, false);
+      if (lane < 6) (lane < 3 ? S.x0.r : S.x1.r)[lane % 3] += dx[lane < 3 ? lane : 14 + lane];
+      __syncwarp();
+      fast_transforms(c, S);          // of no use to anyone should the step fail
     }
   }
   __syncthreads();
-  if (!S.good[0] || !S.good[1]) {
+  if (!S.good) {
     if (tid == 0) c->status = DRI_ELOST;
     return true;
   }
   if (warp == 0) {
-    fast_transforms(c, S);
-  } else if (warp == 1) {
     if (lane < 20) reinterpret_cast<double*>(&c->x0)[lane] = reinterpret_cast<const double*>(&S.x0)[lane];
   } else if (warp == 2) {
     if (lane < 20) reinterpret_cast<double*>(&c->x1)[lane] = reinterpret_cast<const double*>(&S.x1)[lane];
@@ -1117,16 +1143,9 @@ __device__ bool gn_step_fast(const SolveParams& sp, FastSmem& S) {
 // is swept by one warp without block barriers.  Against a block-wide factorisation
 // with FP64 divisions and a one-thread substitution: 18 -> 12 us per step (with its launch), 501x377 camera
 // 495 -> 362 us per frame.
-__device__ void gn_step_pose_only(const SolveParams& sp, FastSmem& S) {
+__device__ void gn_step_pose_only(const SolveParams& sp, FastSmem& S, Ctrl* c, const FastLoad& fl) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  Ctrl* c = sp.ctrl;
-  const int status = c->status;
-  if (tid < 20) reinterpret_cast<double*>(&S.x0)[tid] = reinterpret_cast<const double*>(&c->x0)[tid];
-  else if (tid < 40) reinterpret_cast<double*>(&S.x1)[tid - 20] = reinterpret_cast<const double*>(&c->x1)[tid - 20];
-  else if (tid >= 64 && tid < 73) S.Rref[tid - 64] = c->Rref[tid - 64];
-  else if (tid >= 73 && tid < 76) S.rref[tid - 73] = c->rref[tid - 73];
-  if (status != 0) return;
-  __syncthreads();
+  if (fl.status != 0) return;
   // C: diag(R0, R0) (photometric, rows 0-5) and diag(R_ref, R_ref) (ICP, rows 6-11)
   if (tid < 9) S.R0[tid] = quat_rot_e(S.x0.q, tid);
   __syncwarp();

@@ -2053,19 +2053,22 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_gn_step_batch(const BatchA
   extern __shared__ __align__(16) unsigned char smem_raw[];
   grid_dep_launch();                    // the next pixel kernel waits for this step itself
   const bool lin = (int)blockIdx.x >= a.nslots;        // a frame's last launch has two blocks per slot
-  const int mode = load_slot_params(a, sp, lin ? blockIdx.x - a.nslots : blockIdx.x);
+  const int i = lin ? blockIdx.x - a.nslots : blockIdx.x;
+  Ctrl* c = a.nslots <= kArgCtrls ? a.ctrl[i] : a.slots[a.slot0 + i].sp.ctrl;
+  FastSmem& F = *reinterpret_cast<FastSmem*>(smem_raw);
+  const FastLoad fl = fast_load(c, F);
+  const int mode = load_slot_params(a, sp, i);
   if (mode != kSlotTrack) {
     grid_dep_wait();                    // idle slot: nothing to read, keep the ordering
   } else if (sp.gdof == 3) {
     if (!lin) gn_step_g3(sp, *reinterpret_cast<Gn3Smem*>(smem_raw));
   } else if (sp.track_mode == DRI_TRACK_RGBD_ONLY) {
-    if (!lin) gn_step_pose_only(sp, *reinterpret_cast<FastSmem*>(smem_raw));
+    if (!lin) gn_step_pose_only(sp, F, c, fl);
   } else if (lin) {
     step_lin_block(sp, *reinterpret_cast<GnSmem*>(smem_raw));
   } else {
     // the covariance form, except where the frame's prior does not allow it
-    if (!gn_step_fast(sp, *reinterpret_cast<FastSmem*>(smem_raw)))
-      gn_step_body(sp, *reinterpret_cast<GnSmem*>(smem_raw));
+    if (!gn_step_fast(sp, F, c, fl)) gn_step_body(sp, *reinterpret_cast<GnSmem*>(smem_raw));
   }
 }
 
