@@ -361,9 +361,15 @@ void plan_fill_tables(Plan* p) {
   }
 }
 
-// Pixel-kernel blocks of group g at level l, and the byte offset of its prefix.
+// Pixel-kernel blocks and the most rows per thread of group g at level l, and the byte
+// offset of its prefix.
 int track_blocks(const Plan* p, int l, int g) {
   return p->pre_track[l][p->gfirst[g] + g + p->gcount[g]];
+}
+int track_rows(const Plan* p, int l, int g) {
+  int r = 0;
+  for (int i = p->gfirst[g]; i < p->gfirst[g] + p->gcount[g]; ++i) r = std::max(r, p->ppt[i][l]);
+  return r;
 }
 size_t track_start(const Plan* p, int l, int g) {
   return p->tv.track_off[l] + (size_t)(p->gfirst[g] + g) * sizeof(int32_t);
@@ -716,7 +722,7 @@ int plan_enqueue(Plan* p, int phases, int64_t* kernels) {
           const int nb = track_blocks(p, l, g);
           CK(launch(prof, DRI_KC_TRACK, plan_pixels(p, l) * px_scale,
                     [&] {
-                      return launch_track_batch(at, nb, p->fp16, p->fp32p, p->opt, prio, p->groups == 1, sg);
+                      return launch_track_batch(at, nb, track_rows(p, l, g), p->fp16, p->fp32p, p->opt, prio, p->groups == 1, sg);
                     }));
           const BatchArgs as = plan_args(p, p->tv.copy_off, l, remaining == 0, p->gfirst[g], p->gcount[g]);
           CK(launch(prof, DRI_KC_SOLVE, 0.0, [&] { return launch_gn_step_batch(as, p->g3, sg); }));
@@ -761,7 +767,7 @@ int plan_autotune(Plan* p, int64_t* kernels) {
       auto all_groups = [&] {
         for (int g = 0; g < p->groups; ++g) {
           const BatchArgs at = plan_args(p, track_start(p, l, g), l, 0, p->gfirst[g], p->gcount[g]);
-          if (launch_track_batch(at, track_blocks(p, l, g), p->fp16, p->fp32p, p->opt, launch_priority(false),
+          if (launch_track_batch(at, track_blocks(p, l, g), c, p->fp16, p->fp32p, p->opt, launch_priority(false),
                                  true, p->stream) !=
               cudaSuccess)
             return false;
@@ -1457,7 +1463,7 @@ int dri_linearise(dri_stream s, int32_t level, const dri_state* x0, const dri_st
     af.flags = s->flags;
     CK(cudaMemsetAsync(s->flags, 0, nflags, s->stream));
     CK(launch(s, DRI_KC_TRACK, px, [&] {
-      return launch_track_batch(af, nb, p->fp16, p->fp32p, p->opt, launch_priority(false), false, s->stream);
+      return launch_track_batch(af, nb, p->ppt[0][level], p->fp16, p->fp32p, p->opt, launch_priority(false), false, s->stream);
     }));
     // the flag-writing launch counted the margin decisions too: count once
     CK(cudaMemsetAsync(s->ctrl->margin_acc, 0, sizeof(s->ctrl->margin_acc), s->stream));
@@ -1465,7 +1471,7 @@ int dri_linearise(dri_stream s, int32_t level, const dri_state* x0, const dri_st
   BatchArgs am = at;
   am.margin = 1;                   // the margin decisions, counted as a level's last iteration does
   CK(launch(s, DRI_KC_TRACK, px, [&] {
-    return launch_track_batch(am, nb, p->fp16, p->fp32p, p->opt, launch_priority(false), false, s->stream);
+    return launch_track_batch(am, nb, p->ppt[0][level], p->fp16, p->fp32p, p->opt, launch_priority(false), false, s->stream);
   }));
   CK(launch(s, DRI_KC_SOLVE, 0.0, [&] { return launch_linearise_end(sp, s->lin_dev, s->stream); }));
   s->launches += 1 + 2 * L - 1 + 3 + (flags ? 1 : 0);

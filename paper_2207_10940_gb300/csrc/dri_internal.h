@@ -38,6 +38,7 @@ constexpr int kSumsAll = 2 * kSums;   // ICP then photometric
 constexpr int kTrackThreadsX = 32;
 constexpr int kTrackThreadsY = 8;      // warps of a pixel-kernel block
 constexpr int kTrackRows = 4;          // mixed-term tiles: rows per unit of rows-per-thread
+constexpr int kNumSms = 152;           // GB300
 constexpr int kFoldGroup = 16;        // blocks per first-level fold of the pixel kernel
 
 struct DState {                       // Eq. 1
@@ -313,7 +314,8 @@ int launch_priority(bool solver);
 // early: programmatic dependent launch after the preceding Gauss-Newton step (its
 // blocks then wait on the SMs for the step's end, which only pays when no other
 // slot group could use those SMs meanwhile)
-cudaError_t launch_track_batch(const BatchArgs& a, int blocks, bool fp16, bool fp32_partials, int opt,
+// rows: the most rows per thread of the launch's slots
+cudaError_t launch_track_batch(const BatchArgs& a, int blocks, int rows, bool fp16, bool fp32_partials, int opt,
                                int priority, bool early, cudaStream_t s);
 int track_grid_blocks(int w, int h, int ppt);   // batched kernel: single-term blocks
 int track_mixed_blocks(int w, int h, int ppt);  // by-value kernel: mixed-term blocks

@@ -665,8 +665,8 @@ k_track(TrackParams p, const __grid_constant__ PairEnd end) {
 // more spill reloads) and than two columns per thread.
 // FLAGS (parity entry only): the same kernel that also or-s each pixel's
 // validity bits into a.flags (the slot's level image, zeroed before the launch).
-template <typename T, typename P, int OPT, bool FLAGS, bool MARGIN>
-__global__ void __launch_bounds__(kTrackThreadsX * kTrackThreadsY, 3)
+template <typename T, typename P, int OPT, bool FLAGS, bool MARGIN, int BLOCKS>
+__global__ void __launch_bounds__(kTrackThreadsX * kTrackThreadsY, BLOCKS)
 k_track_batch(const BatchArgs a) {
   const int i = batch_slot(a, blockIdx.x);
   const int slot = a.slot0 + i;
@@ -751,7 +751,7 @@ cudaError_t launch_track(const TrackParams& p0, const PairEnd& end, bool fp16, b
 #undef DRI_TRACK_OPT
 }
 
-cudaError_t launch_track_batch(const BatchArgs& a, int blocks, bool fp16, bool fp32_partials,
+cudaError_t launch_track_batch(const BatchArgs& a, int blocks, int rows, bool fp16, bool fp32_partials,
                                int opt, int priority, bool early, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(blocks);
@@ -764,18 +764,26 @@ cudaError_t launch_track_batch(const BatchArgs& a, int blocks, bool fp16, bool f
   attr[1].val.priority = priority;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-#define DRI_TRACK_BATCH_F(T, P, F, M)                                                    \
+  // A launch that nothing else shares the GPU with and that is a little larger than one
+  // wave at three blocks per SM runs at four (64 registers, some spills) when its tiles
+  // are short: the second wave would hold back the step behind it, which starts once
+  // every block has started (600 blocks of one row: 320x240 488 -> 462 us per frame,
+  // 640x480 575 -> 562).  With long tiles the spills cost more than the wave (480 blocks
+  // of 16 rows: 1277x717 725 -> 801, 12 x 320x240 836 -> 910).
+  const bool four = early && rows <= 2 && blocks > 3 * kNumSms && blocks <= 4 * kNumSms;
+#define DRI_TRACK_BATCH_F(T, P, F, M, B)                                                 \
   do {                                                                                   \
-    if (opt == 0) return cudaLaunchKernelEx(&cfg, k_track_batch<T, P, 0, F, M>, a);      \
-    if (opt == 1) return cudaLaunchKernelEx(&cfg, k_track_batch<T, P, 1, F, M>, a);      \
-    if (opt == 2) return cudaLaunchKernelEx(&cfg, k_track_batch<T, P, 2, F, M>, a);      \
-    return cudaLaunchKernelEx(&cfg, k_track_batch<T, P, 3, F, M>, a);                    \
+    if (opt == 0) return cudaLaunchKernelEx(&cfg, k_track_batch<T, P, 0, F, M, B>, a);   \
+    if (opt == 1) return cudaLaunchKernelEx(&cfg, k_track_batch<T, P, 1, F, M, B>, a);   \
+    if (opt == 2) return cudaLaunchKernelEx(&cfg, k_track_batch<T, P, 2, F, M, B>, a);   \
+    return cudaLaunchKernelEx(&cfg, k_track_batch<T, P, 3, F, M, B>, a);                 \
   } while (0)
 #define DRI_TRACK_BATCH(T, P)                                                            \
   do {                                                                                   \
-    if (a.flags) DRI_TRACK_BATCH_F(T, P, true, true);                                    \
-    if (a.margin) DRI_TRACK_BATCH_F(T, P, false, true);                                  \
-    DRI_TRACK_BATCH_F(T, P, false, false);                                               \
+    if (a.flags) DRI_TRACK_BATCH_F(T, P, true, true, 3);                                 \
+    if (a.margin) DRI_TRACK_BATCH_F(T, P, false, true, 3);                               \
+    if (four) DRI_TRACK_BATCH_F(T, P, false, false, 4);                                  \
+    DRI_TRACK_BATCH_F(T, P, false, false, 3);                                            \
   } while (0)
   if (fp16) {
     if (fp32_partials) DRI_TRACK_BATCH(__half, float);
