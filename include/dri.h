@@ -279,7 +279,7 @@ int dri_track(dri_stream s, dri_track_result* out);
 
 /* Tracks the uploaded frame of each of n streams (Sec. IV, as dri_track) in
  * one batched launch sequence: every kernel of a frame (maps, frame start, each
- * Gauss-Newton iteration's pixel kernel and solve, marginalisation, gradients)
+ * Gauss-Newton iteration's pixel kernel and solve, marginalisation)
  * is one launch over the pixels or states of all n streams.  The paper tracks
  * one camera; batching independent streams is this library's throughput mode.
  *
@@ -456,11 +456,11 @@ int dri_io_bytes(dri_stream s, int64_t* h2d, int64_t* d2h);
 /* Per-kernel-class device time, measured with CUDA events recorded on the
  * stream around each launch while profiling is enabled (tracing aid; adds two
  * event records per launch).  Classes: */
-#define DRI_KC_MAPS     0   /* level-0 copy, pyramid downsample, normal maps      */
+#define DRI_KC_MAPS     0   /* pyramid, normal and intensity-gradient maps        */
 #define DRI_KC_TRACK    1   /* fused photometric + ICP linearisation and reduction */
 #define DRI_KC_SOLVE    2   /* Gauss-Newton step (IMU, assembly, Cholesky, update) */
 #define DRI_KC_FRAME    3   /* frame begin / end / init (IMU weight, Schur)        */
-#define DRI_KC_GRAD     4   /* reference intensity-gradient maps                   */
+#define DRI_KC_GRAD     4   /* stays 0: gradients are built with the normal maps   */
 #define DRI_KC_COUNT    8
 typedef struct {
     int64_t launches[DRI_KC_COUNT];

@@ -396,7 +396,6 @@ void plan_free(Plan* p) {
   for (cudaStream_t a : p->aux)
     if (a) cudaStreamDestroy(a);
   if (p->ev_fork) cudaEventDestroy(p->ev_fork);
-  if (p->ev_grad) cudaEventDestroy(p->ev_grad);
   if (p->ev_maps) cudaEventDestroy(p->ev_maps);
   if (p->ev_start) cudaEventDestroy(p->ev_start);
   if (p->ev_begin) cudaEventDestroy(p->ev_begin);
@@ -480,7 +479,6 @@ int plan_create(dri_stream_s* const* streams, int n, int ring, bool in_workspace
   p->ev_join.assign(kMaxGroups - 1, nullptr);
   if (!in_workspace) {
     if (cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&p->ev_grad, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&p->ev_maps, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&p->ev_start, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&p->ev_begin, cudaEventDisableTiming) != cudaSuccess ||
@@ -630,13 +628,13 @@ cudaStream_t side_stream(const Plan* p, bool profiling) {
 }
 
 // Kernel launches of one frame, in order.  phase 1: maps and frame begin;
-// phase 2: the Gauss-Newton loop, frame end, gradients and the head gather.
+// phase 2: the Gauss-Newton loop, frame end and the head gather.
 // On the plan's spare stream: the frame start, beside the map kernels
 // (it reads and writes the slots' control blocks and their IMU blocks, the map
 // kernels only which set is the reference, which changes at the frame end),
-// and beside the loop the normal maps of the finer levels (the loop starts at
-// the coarsest; each group waits for them before its first finer-level pixel
-// kernel) and the gradient maps.
+// and beside the loop the normal and gradient maps of the finer levels (the loop
+// starts at the coarsest; each group waits for them before its first finer-level
+// pixel kernel).
 int plan_enqueue(Plan* p, int phases, int64_t* kernels) {
   dri_stream_s* prof = p->slots[0];
   cudaStream_t st = p->stream;
@@ -655,14 +653,8 @@ int plan_enqueue(Plan* p, int phases, int64_t* kernels) {
     }
     const BatchArgs a0 = plan_args(p, p->tv.copy_off, 0, 0);
     CK(launch(prof, DRI_KC_MAPS, plan_pixels(p, 0),
-              [&] { return launch_copy_batch(a0, p->pre_copy[p->S], st); }));
+              [&] { return launch_pyramid_batch(a0, p->pre_copy[p->S], st); }));
     ++k;
-    for (int l = 1; l < L; ++l) {
-      const BatchArgs a = plan_args(p, p->tv.map_off[l], l, 0);
-      CK(launch(prof, DRI_KC_MAPS, plan_pixels(p, l),
-                [&] { return launch_pyr_down_batch(a, p->pre_map[l][p->S], st); }));
-      ++k;
-    }
     p->norm_side = sside != st && L > 1;
     if (p->norm_side) {
       CK(cudaEventRecord(p->ev_maps, st));
@@ -672,7 +664,7 @@ int plan_enqueue(Plan* p, int phases, int64_t* kernels) {
       const BatchArgs a = plan_args(p, p->tv.map_off[l], l, 0);
       const cudaStream_t sn = (p->norm_side && l < L - 1) ? sside : st;
       CK(launch(prof, DRI_KC_MAPS, plan_pixels(p, l),
-                [&] { return launch_normals_batch(a, p->pre_map[l][p->S], p->fp16, sn); }));
+                [&] { return launch_maps_batch(a, p->pre_map[l][p->S], p->fp16, sn); }));
       ++k;
     }
     if (p->norm_side) CK(cudaEventRecord(p->ev_norm, sside));
@@ -693,19 +685,7 @@ int plan_enqueue(Plan* p, int phases, int64_t* kernels) {
     // of 16 x 640x480: 7.4k frames/s early, 12.3k not).  While profiling, the
     // groups run one after the other on the plan's stream.
     const bool fork = p->groups > 1 && !prof->profiling;
-    // The gradient maps of the frame's own set (the next reference's pack B)
-    // depend on its intensity pyramid only: they run on a spare stream beside
-    // the Gauss-Newton loop and are joined before the frame end.
-    const cudaStream_t sgrad = sside;
-    if (fork || sgrad != st) CK(cudaEventRecord(p->ev_fork, st));
-    if (sgrad != st) CK(cudaStreamWaitEvent(sgrad, p->ev_fork, 0));
-    for (int l = 0; l < L; ++l) {
-      const BatchArgs a = plan_args(p, p->tv.map_off[l], l, 0);
-      CK(launch(prof, DRI_KC_GRAD, plan_pixels(p, l),
-                [&] { return launch_gradient_batch(a, p->pre_map[l][p->S], p->fp16, sgrad); }));
-      ++k;
-    }
-    if (sgrad != st) CK(cudaEventRecord(p->ev_grad, sgrad));
+    if (fork) CK(cudaEventRecord(p->ev_fork, st));
     for (int g = 0; g < p->groups; ++g) {
       cudaStream_t sg = (fork && g > 0) ? p->aux[g - 1] : st;
       if (fork && g > 0) CK(cudaStreamWaitEvent(sg, p->ev_fork, 0));
@@ -734,7 +714,6 @@ int plan_enqueue(Plan* p, int phases, int64_t* kernels) {
         CK(cudaStreamWaitEvent(st, p->ev_join[g - 1], 0));
       }
     }
-    if (sgrad != st) CK(cudaStreamWaitEvent(st, p->ev_grad, 0));
     const BatchArgs ae = plan_args(p, p->tv.copy_off, 0, 0);
     CK(launch(prof, DRI_KC_FRAME, 0.0, [&] { return launch_frame_end_batch(ae, st); }));
     ++k;
@@ -804,9 +783,9 @@ int plan_autotune(Plan* p, int64_t* kernels) {
 // The spare stream and its events of a stream's own plan, held only while its launch
 // sequence is captured: the graph keeps the branches (one 640x480 camera 743 -> 667 us
 // per frame against one chain: the frame start beside the map kernels, the finer
-// levels' normals and the gradients beside the loop).
+// levels' maps beside the loop).
 void free_capture_side(Plan* p) {
-  cudaEvent_t* ev[] = {&p->ev_fork, &p->ev_grad, &p->ev_maps, &p->ev_start, &p->ev_begin, &p->ev_norm};
+  cudaEvent_t* ev[] = {&p->ev_fork, &p->ev_maps, &p->ev_start, &p->ev_begin, &p->ev_norm};
   for (cudaEvent_t* e : ev) {
     if (*e) cudaEventDestroy(*e);
     *e = nullptr;
@@ -816,7 +795,7 @@ void free_capture_side(Plan* p) {
 }
 
 void make_capture_side(Plan* p) {
-  cudaEvent_t* ev[] = {&p->ev_fork, &p->ev_grad, &p->ev_maps, &p->ev_start, &p->ev_begin, &p->ev_norm};
+  cudaEvent_t* ev[] = {&p->ev_fork, &p->ev_maps, &p->ev_start, &p->ev_begin, &p->ev_norm};
   bool ok = cudaStreamCreateWithFlags(&p->aux[kMaxGroups - 2], cudaStreamNonBlocking) == cudaSuccess;
   for (cudaEvent_t* e : ev) ok = ok && cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
   if (!ok) {                      // without it the sequence is captured as one chain
@@ -1436,15 +1415,11 @@ int dri_linearise(dri_stream s, int32_t level, const dri_state* x0, const dri_st
   // the maps of the pending frame (the frame itself stays pending)
   const int L = s->cfg.levels;
   const BatchArgs a0 = plan_args(p, p->tv.copy_off, 0, 0);
-  CK(launch(s, DRI_KC_MAPS, 0.0, [&] { return launch_copy_batch(a0, p->pre_copy[1], s->stream); }));
-  for (int l = 1; l < L; ++l) {
-    const BatchArgs a = plan_args(p, p->tv.map_off[l], l, 0);
-    CK(launch(s, DRI_KC_MAPS, 0.0, [&] { return launch_pyr_down_batch(a, p->pre_map[l][1], s->stream); }));
-  }
+  CK(launch(s, DRI_KC_MAPS, 0.0, [&] { return launch_pyramid_batch(a0, p->pre_copy[1], s->stream); }));
   for (int l = 0; l < L; ++l) {
     const BatchArgs a = plan_args(p, p->tv.map_off[l], l, 0);
     CK(launch(s, DRI_KC_MAPS, 0.0,
-              [&] { return launch_normals_batch(a, p->pre_map[l][1], p->fp16, s->stream); }));
+              [&] { return launch_maps_batch(a, p->pre_map[l][1], p->fp16, s->stream); }));
   }
   const SolveParams sp = solve_params(s, level, 0);
   CK(launch(s, DRI_KC_FRAME, 0.0,
@@ -1474,7 +1449,7 @@ int dri_linearise(dri_stream s, int32_t level, const dri_state* x0, const dri_st
     return launch_track_batch(am, nb, p->ppt[0][level], p->fp16, p->fp32p, p->opt, launch_priority(false), false, s->stream);
   }));
   CK(launch(s, DRI_KC_SOLVE, 0.0, [&] { return launch_linearise_end(sp, s->lin_dev, s->stream); }));
-  s->launches += 1 + 2 * L - 1 + 3 + (flags ? 1 : 0);
+  s->launches += 1 + L + 3 + (flags ? 1 : 0);
   CK(cudaMemcpyAsync(out, s->lin_dev, sizeof(*out), cudaMemcpyDeviceToHost, s->stream));
   if (flags) CK(cudaMemcpyAsync(flags, s->flags, nflags, cudaMemcpyDeviceToHost, s->stream));
   CK(cudaMemcpyAsync(s->pin_ctrl, s->ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s->stream));

@@ -177,9 +177,9 @@ struct SolveParams {
 // ---- batched launches --------------------------------------------------------
 enum SlotMode : int32_t { kSlotIdle = 0, kSlotTrack = 1, kSlotInit = 2 };
 
-constexpr int kCopyTileW = 128;       // level-0 input copy: 32 x 8 threads, 4 pixels each
-constexpr int kCopyTileH = 8;
-constexpr int kMapTileW = 32;         // pyramid, normal and gradient maps: 32 x 8 threads
+constexpr int kCopyTileW = 64;        // level-0 copy and pyramid: 32 x 8 threads of 2 x 4 pixels
+constexpr int kCopyTileH = 32;
+constexpr int kMapTileW = 32;         // normal and gradient maps: 32 x 8 threads
 constexpr int kMapTileH = 8;          // block rows; a thread takes kMapRows rows of its tile
 constexpr int kMapRows = 8;           // 32 x 64 tiles: 8 rows per thread measured 1.4-1.6x faster
                                       // than one (block scheduling dominated 256-pixel blocks)
@@ -263,10 +263,8 @@ struct RefUpload {
 cudaError_t launch_upload_reference(const LevelMaps* m, const LevelGeom* g, int levels, Ctrl* ctrl,
                                     float dmin, float dmax, bool fp16, const RefUpload& up,
                                     cudaStream_t s);
-cudaError_t launch_copy_batch(const BatchArgs& a, int blocks, cudaStream_t s);
-cudaError_t launch_pyr_down_batch(const BatchArgs& a, int blocks, cudaStream_t s);
-cudaError_t launch_normals_batch(const BatchArgs& a, int blocks, bool fp16, cudaStream_t s);
-cudaError_t launch_gradient_batch(const BatchArgs& a, int blocks, bool fp16, cudaStream_t s);
+cudaError_t launch_pyramid_batch(const BatchArgs& a, int blocks, cudaStream_t s);
+cudaError_t launch_maps_batch(const BatchArgs& a, int blocks, bool fp16, cudaStream_t s);
 inline int copy_tiles(int w, int h) {
   return ((w + kCopyTileW - 1) / kCopyTileW) * ((h + kCopyTileH - 1) / kCopyTileH);
 }
