@@ -767,8 +767,8 @@ cudaError_t launch_track_batch(const BatchArgs& a, int blocks, int rows, bool fp
   // A launch that nothing else shares the GPU with and that is a little larger than one
   // wave at three blocks per SM runs at four (64 registers, some spills) when its tiles
   // are short: the second wave would hold back the step behind it, which starts once
-  // every block has started (600 blocks of one row: 320x240 488 -> 462 us per frame,
-  // 640x480 575 -> 562).  With long tiles the spills cost more than the wave (480 blocks
+  // every block has started (600 blocks of one row: 320x240 490 -> 465 us per frame,
+  // 640x480 591 -> 577).  With long tiles the spills cost more than the wave (480 blocks
   // of 16 rows: 1277x717 725 -> 801, 12 x 320x240 836 -> 910).
   const bool four = early && rows <= 2 && blocks > 3 * kNumSms && blocks <= 4 * kNumSms;
 #define DRI_TRACK_BATCH_F(T, P, F, M, B)                                                 \
