@@ -41,6 +41,11 @@
 // Included by solve.cu, inside its namespace, after the element-wise 3x3 algebra
 // and the warp-cooperative state algebra that it uses.
 
+// Named barriers.  The ids of a step: 1 warps 0-3 and 3 warps 4-7 among themselves, 5
+// warps 0-2, 6 warps 1-2; hand-offs (one side arrives and goes on, the other waits) 4
+// pixel terms, 7 errors, 8 position rows, 9 poses.  A hand-off keeps an id of its own:
+// the arriving warp may come back to a shared one before the waiting warps have passed
+// it, and would be counted twice.
 template <int ID, int N>
 __device__ __forceinline__ void bar_sync() { asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(N) : "memory"); }
 template <int ID, int N>
@@ -823,7 +828,7 @@ __device__ bool gn_step_fast(const SolveParams& sp, FastSmem& S, Ctrl* c, const 
         for (int i = lane; i < 33; i += 32) S.Jyr[i / 11][i % 11] = 0.0;
         __syncwarp();
       }
-      bar_arrive<5, 96>();
+      bar_arrive<8, 96>();            // the position rows to warps 1 and 2
       // e_a = log(M): the skew part v = 2 sin(t) k, t / (2 sin t) from its series in
       // sin^2 t (the angle is below 6.4 mrad in all but a frame's first iterations)
       double ea;
@@ -868,7 +873,7 @@ __device__ bool gn_step_fast(const SolveParams& sp, FastSmem& S, Ctrl* c, const 
       }
     }
     if (warp == 1 || warp == 2) {     // position rows: Jy P, Jp + Jy K, e + Jy m
-      bar_sync<5, 96>();
+      bar_sync<8, 96>();
       const int q = lane - 11;
       const int r = warp == 1 ? lane / 11 : lane < 11 ? 2 : lane < 29 ? q / 6 : lane - 29;
       const int cc = warp == 1 ? lane - 11 * r : lane < 11 ? lane : lane < 29 ? q - 6 * r : 0;
@@ -1031,7 +1036,7 @@ __device__ bool gn_step_fast(const SolveParams& sp, FastSmem& S, Ctrl* c, const 
         dx[lane < kLam + 6 ? lane - kLam : 4 + lane] = y;     // p0 at 0..5, p1 at 17..22
       }
       __syncwarp();
-      bar_arrive<6, 64>();
+      bar_arrive<9, 64>();
       substitute(kLam, 0);
       if (lane < kLam) S.z[lane] = y;
       __syncwarp();
@@ -1104,7 +1109,7 @@ __device__ bool gn_step_fast(const SolveParams& sp, FastSmem& S, Ctrl* c, const 
         (f == 0 ? x.v : f == 1 ? x.bg : x.ba)[i - 3 * f] += dx[17 * q + 6 + i];
       }
     } else if (warp == 1) {
-      bar_sync<6, 64>();
+      bar_sync<9, 64>();
       fast_quat_boxplus(S.x0.q, dx + 3, false, S.x1.q, dx + 20, false);
       if (lane < 6) (lane < 3 ? S.x0.r : S.x1.r)[lane % 3] += dx[lane < 3 ? lane : 14 + lane];
       __syncwarp();
