@@ -530,7 +530,10 @@ __device__ __forceinline__ bool track_tile(const TrackParams& p, const int term,
   else rgb_rows<T, (OPT & kOptOcc) != 0, FLAGS, MARGIN>(c, acc, nm);
   if (MARGIN) {                      // the warp's margin decisions, one integer add
     const unsigned sum = __reduce_add_sync(0xffffffffu, (unsigned)nm);
-    if (lane == 0 && sum) atomicAdd(&ctrl->margin_acc[icp ? 0 : 1], sum);
+    if (lane == 0 && sum) {
+      atomicAdd(&ctrl->margin_acc[icp ? 0 : 1], sum);
+      if (!SPLIT) __threadfence();   // the pair kernel's last block reads them: before this block counts as done
+    }
   }
 
   // ---------------- reduction ----------------
