@@ -1753,12 +1753,14 @@ __device__ void frame_begin_body(const SolveParams& sp, BeginSmem& B) {
 
 // The state-only part of the joint system at the last iteration's linearisation point
 // (c->xl0, c->xl1), for the marginalisation: a block of its own beside the step's, whose
-// covariance form does not produce it.  Nothing it reads is written by that step (the
-// first-order update's linearisation point does not move in a frame's last step).
+// covariance form does not produce it.  Of what it reads that step writes the status only
+// (the first-order update's linearisation point does not move in a frame's last step): a
+// step that fails beside it may be seen by some threads and not by others, so the block
+// decides as one.  Where it goes on regardless, nobody uses what it leaves.
 __device__ void step_lin_block(const SolveParams& sp, GnSmem& S) {
   Ctrl* c = sp.ctrl;
   const int tid = threadIdx.x;
-  if (c->status != 0 || !c->elim.ok) return;
+  if (__syncthreads_or(c->status != 0 || !c->elim.ok)) return;
   assemble_state(sp, S, c->xl0, c->xl1, false);
   if (!S.ok) return;                  // the step itself reports it
   for (int idx = tid; idx < 34 * 34; idx += kSolveThreads) {

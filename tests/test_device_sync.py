@@ -27,3 +27,15 @@ def test_hand_off_barriers_have_an_id_of_their_own():
             found += 1
             assert len(counts) == 1 and sync.get(bid) == counts, (name, bid, counts, sync.get(bid))
     assert found >= 4
+
+
+def test_a_block_that_shares_its_launch_with_the_step_decides_as_one():
+    """The block that assembles the last system reads the camera's status, which the
+    step's block of the same launch may be writing: its threads must not each decide by
+    what they happened to read (the code behind the test has block barriers)."""
+    text = dict(sources())["solve.cu"]
+    body = text[text.index("void step_lin_block("):]
+    body = body[:body.index("\n}")]
+    tests = re.findall(r"if \(([^;]*)\) return;", body)
+    assert any("status" in t for t in tests)
+    assert all(t.startswith("__syncthreads_or(") for t in tests if "status" in t), tests
