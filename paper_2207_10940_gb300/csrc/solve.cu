@@ -1899,9 +1899,9 @@ __device__ void frame_end_body(const SolveParams& sp, EndSmem& E) {
       }
       __syncthreads();
     }
+    const unsigned m = __ballot_sync(0xffffffffu, tid < 4 * NJ);
     if (tid < 4 * NJ) {               // b' = b - H d, four lanes per row
       const int i = tid >> 2, q = tid & 3;
-      const unsigned m = __activemask();
       double v = 0.0;
       for (int k = q; k < NJ; k += 4) v = fma(-E.H[i * NJ + k], E.d[k], v);
       v += __shfl_xor_sync(m, v, 1);

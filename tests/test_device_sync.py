@@ -39,3 +39,10 @@ def test_a_block_that_shares_its_launch_with_the_step_decides_as_one():
     tests = re.findall(r"if \(([^;]*)\) return;", body)
     assert any("status" in t for t in tests)
     assert all(t.startswith("__syncthreads_or(") for t in tests if "status" in t), tests
+
+
+def test_shuffle_masks_are_not_taken_from_the_running_threads():
+    """__activemask() names the threads that happen to run together, which need not be
+    all that a branch holds; a mask for the branch is taken by a ballot before it."""
+    for name, text in sources():
+        assert "__activemask" not in text, name
