@@ -1198,7 +1198,7 @@ __device__ void gn_step_pose_only(const SolveParams& sp, FastSmem& S, Ctrl* c, c
       *(j == k ? cb + i : S.sink + lane) = v;
       __syncwarp();
       const double t = cb[max(i, 0)] * cb[max(j, 0)];
-      const double r = pivot_recip(cb[k]);
+      const double r = pivot_recip<true>(cb[k]);
       const double w = fma(-t, r, v);
       v = j > k ? w : v;
       rown = j == k ? r : rown;
@@ -1232,13 +1232,6 @@ __device__ void gn_step_pose_only(const SolveParams& sp, FastSmem& S, Ctrl* c, c
 }
 
 // ---- the frame's constants (k_frame_begin) -----------------------------------------
-
-// Reciprocal of a positive pivot to FP64 rounding (two Newton steps): the frame's
-// constants and the marginalisation subtract large terms from one another.
-__device__ __forceinline__ double pivot_recip_full(double d) {
-  const double y = pivot_recip(d);
-  return fma(y, fma(-d, y, 1.0), y);
-}
 
 // Entry (i, j) of a symmetric matrix after the sweep operator on index k: -1 / d on the
 // pivot, a / d in its row and column, a - c_i c_j / d elsewhere; c: column k, r = 1 / d.
@@ -1315,7 +1308,7 @@ __device__ void prepare_elim(const SolveParams& sp, Ctrl* c, int np, const doubl
       if (i == k && j == k && !(v[o] > 1e-12 * diag[o] && v[o] < 1e29)) *bad = 1;
     }
     bar_sync<1, 128>();
-    const double r = pivot_recip_full(ck[k]);
+    const double r = pivot_recip<true>(ck[k]);
 #pragma unroll
     for (int o = 0; o < 2; ++o) v[o] = sweep_entry(ei[o], ej[o], k, v[o], ck, r);
   }

@@ -715,6 +715,11 @@ __device__ void warp_write_transforms(Ctrl* c, const DState& x0, const DState& x
 // formats; d and 1 / d are normal in both here) and the seed itself is the
 // hardware's approximation: on this GPU every FP64-pipe instruction on the
 // pivot's dependency chain, a comparison included, costs 64 cycles.
+// FULL: to FP64 rounding, by one step of third order (Householder's: with e = 1 - d y,
+// y (1 + e + e^2), error e^3 < 2^-67) instead of second, which is one dependent
+// operation more: the RGB-D-only step's system is solved to rounding, and the frame's
+// constants and the marginalisation subtract large terms from one another.
+template <bool FULL = false>
 __device__ __forceinline__ double pivot_recip(double d) {
   const int hi = __double2hiint(d);
   if ((unsigned)((hi >> 20) - (1023 - 99)) < 198u) {       // 2^-99 <= d < 2^99, positive
@@ -724,7 +729,8 @@ __device__ __forceinline__ double pivot_recip(double d) {
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(__uint_as_float(fb)));
     const int yb = __float_as_int(y0);
     const double y = __hiloint2double((yb >> 3) + 0x38000000, (int)((unsigned)yb << 29));
-    return fma(y, fma(-d, y, 1.0), y);
+    const double e = fma(-d, y, 1.0);
+    return fma(y, FULL ? fma(e, e, e) : e, y);
   }
   return 1.0 / d;
 }
@@ -1670,7 +1676,7 @@ __device__ bool imu_weight_and_prediction(const SolveParams& sp, Ctrl* c, BeginS
       bar_sync<2, 64>();
       const double d = ck[k];
       good = good && __double2hiint(d) > 0 && finite_bits(d);
-      v = sweep_entry(i, j, k, v, ck, pivot_recip_full(d));
+      v = sweep_entry(i, j, k, v, ck, pivot_recip<true>(d));
     }
     if (i >= 0) B.Winv[i * 9 + j] = B.Winv[j * 9 + i] = -v;
     if (t == 0) B.fail = !good;
@@ -1825,7 +1831,7 @@ __device__ bool eliminate_x0(EndSmem& E, Ctrl* c, bool gyro) {
     bar_sync<1, 128>();
     const double d = cb[k];
     good = good && __double2hiint(d) > 0 && finite_bits(d);
-    const double r = pivot_recip_full(d);
+    const double r = pivot_recip<true>(d);
 #pragma unroll
     for (int o = 0; o < kOwn; ++o)
       if (life[o] > k) {              // uniform over the warp
