@@ -1288,7 +1288,7 @@ __device__ void prepare_elim(const SolveParams& sp, Ctrl* c, int np, const doubl
       if (e < 153 && tri(i + 1, 0) <= e) ++i;
       if (e < 153 && tri(i, 0) > e) --i;
       j = e - tri(i, 0);
-      x = i < 17 ? c->Hs[i * 17 + j] : c->bs[j];
+      x = i < 17 ? c->Hs[j * 17 + i] : c->bs[j];     // upper triangle, as assemble_state
       if (gyro && ((i < 17 && held_gyro_only(i)) || held_gyro_only(j))) x = 0.0;
     }
     ei[o] = i;
