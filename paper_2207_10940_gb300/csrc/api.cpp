@@ -371,6 +371,10 @@ int track_rows(const Plan* p, int l, int g) {
   for (int i = p->gfirst[g]; i < p->gfirst[g] + p->gcount[g]; ++i) r = std::max(r, p->ppt[i][l]);
   return r;
 }
+// Whether the loop's pixel kernels are launched early (launch_track_batch): with one slot
+// group, whose SMs nothing else could use meanwhile.  It also selects the kernel's
+// variant, so the tuner times with the same choice.
+bool track_early(const Plan* p) { return p->groups == 1; }
 size_t track_start(const Plan* p, int l, int g) {
   return p->tv.track_off[l] + (size_t)(p->gfirst[g] + g) * sizeof(int32_t);
 }
@@ -702,7 +706,7 @@ int plan_enqueue(Plan* p, int phases, int64_t* kernels) {
           const int nb = track_blocks(p, l, g);
           CK(launch(prof, DRI_KC_TRACK, plan_pixels(p, l) * px_scale,
                     [&] {
-                      return launch_track_batch(at, nb, track_rows(p, l, g), p->fp16, p->fp32p, p->opt, prio, p->groups == 1, sg);
+                      return launch_track_batch(at, nb, track_rows(p, l, g), p->fp16, p->fp32p, p->opt, prio, track_early(p), sg);
                     }));
           const BatchArgs as = plan_args(p, p->tv.copy_off, l, remaining == 0, p->gfirst[g], p->gcount[g]);
           CK(launch(prof, DRI_KC_SOLVE, 0.0, [&] { return launch_gn_step_batch(as, p->g3, sg); }));
@@ -747,7 +751,7 @@ int plan_autotune(Plan* p, int64_t* kernels) {
         for (int g = 0; g < p->groups; ++g) {
           const BatchArgs at = plan_args(p, track_start(p, l, g), l, 0, p->gfirst[g], p->gcount[g]);
           if (launch_track_batch(at, track_blocks(p, l, g), c, p->fp16, p->fp32p, p->opt, launch_priority(false),
-                                 true, p->stream) !=
+                                 track_early(p), p->stream) !=
               cudaSuccess)
             return false;
         }
