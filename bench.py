@@ -514,8 +514,7 @@ def initial_state_at(seq, i):
 def kernel_classes(prof, dri):
     return {name: {"launches": int(prof.launches[c]), "ms": round(prof.ms[c], 4)}
             for name, c in (("maps", dri.DRI_KC_MAPS), ("track", dri.DRI_KC_TRACK),
-                            ("solve", dri.DRI_KC_SOLVE), ("frame", dri.DRI_KC_FRAME),
-                            ("grad", dri.DRI_KC_GRAD))}
+                            ("solve", dri.DRI_KC_SOLVE), ("frame", dri.DRI_KC_FRAME))}
 
 
 def bytes_per_pixel_iter(flags):

@@ -1146,8 +1146,8 @@ __device__ bool gn_step_fast(const SolveParams& sp, FastSmem& S, Ctrl* c, const 
 // other components unchanged.  Whole block; what needs no pixel sum is done before the
 // wait for the pixel kernel, and the 6 x 6 system (27 entries with its right-hand side)
 // is swept by one warp without block barriers.  Against a block-wide factorisation
-// with FP64 divisions and a one-thread substitution: 18 -> 12 us per step (with its launch), 501x377 camera
-// 495 -> 362 us per frame.
+// with FP64 divisions and a one-thread substitution: 18 -> 12 us per step (with its launch),
+// 501x377 camera 495 -> 361 us per frame.
 __device__ void gn_step_pose_only(const SolveParams& sp, FastSmem& S, Ctrl* c, const FastLoad& fl) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (fl.status != 0) return;

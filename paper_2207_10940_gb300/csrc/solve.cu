@@ -2,13 +2,16 @@
 //
 //   frame_begin   x0 := x; IMU pre-integration at x0's biases with the propagated
 //                 noise covariance; W_IMU = Sigma^-1; x1 := the IMU prediction x^1(x0)
-//   gn_step       one Gauss-Newton iteration, in one of two forms: the covariance
-//                 form (joint_step.cuh) for all but a frame's last one, and the
-//                 information form below, which also leaves the full system for
-//                 the marginalisation: re-integrate the IMU at x0's current biases, IMU error (Eq. 5) and its analytic 18x34 Jacobian; rotate
-//                 the pixel kernel's photometric / ICP systems into W and map the
+//   gn_step       one Gauss-Newton iteration: re-integrate the IMU at x0's current
+//                 biases, IMU error (Eq. 5) and its analytic Jacobian; rotate the
+//                 pixel kernel's photometric / ICP systems into W and map the
 //                 photometric one onto both poses; add the prior (Eq. 6/9); solve the
-//                 34x34 system of Eq. 7; x0, x1 boxplus= dx (Eq. 2)
+//                 system of Eq. 7; x0, x1 boxplus= dx (Eq. 2).  All of a frame's
+//                 iterations run in the covariance form (joint_step.cuh), beside
+//                 whose last one a second block assembles the full system for the
+//                 marginalisation (step_lin_block), or, where the frame's pieces
+//                 or prior do not allow that, in the information form below, which
+//                 leaves that system itself
 //   frame_end     marginalise x0 by the Schur complement (Eq. 8) at the updated point,
 //                 make the frame the reference (flip of the map sets)
 //   frame_init    first frame (run by the frame-end kernel): first-frame prior, the
@@ -33,8 +36,8 @@
 // to the end of the interval (state-transition blocks from suffix sums of u_k dt_k
 // and u_k w_k).  These equal the sequential recursion exactly (same algebra,
 // other rounding order).  W_IMU's block structure (a 9x9 block and a diagonal)
-// is used in the assembly.  The step solves the reduced 26-dimensional system
-// (x1's biases and gravity eliminated in closed form) with an element-parallel
+// is used in the assembly.  The information form solves the reduced 26-dimensional
+// system (x1's biases and gravity eliminated in closed form) with an element-parallel
 // LDL^T on four warps; its 14 components that no pixel term touches are
 // eliminated before the pixel sums arrive, the 12 pose components after
 // (gn_step_body).  The 3-D gravity form solves its whole 36-dimensional system.

@@ -420,10 +420,6 @@ __device__ __forceinline__ void rgb_rows(const TileCtx& c, float* acc, int& nm) 
   }
 }
 
-// (true in the block that folded the image's last group and wrote ctrl->sums)
-// One tile of one image (single-term: 32 x 8 * ppt pixels of `term`; mixed:
-// 32 x 4 * ppt pixels, warps 0-3 ICP and 4-7 photometric): (bx, by) its tile
-// coordinates, bid its index in the image's fold order.
 // Optional terms, compile-time variants of the pixel kernels (OPT bits): the
 // photometric occlusion test and the depth-dependent ICP weight.
 constexpr int kOptOcc = 1, kOptDepthWeight = 2;
@@ -471,6 +467,10 @@ __device__ __forceinline__ P fold_partials(const P* __restrict__ src, int n, int
   }
 }
 
+// One tile of one image (single-term: 32 x 8 * ppt pixels of `term`; mixed:
+// 32 x 4 * ppt pixels, warps 0-3 ICP and 4-7 photometric): (bx, by) its tile
+// coordinates, bid its index in the image's fold order.  True in the block that folded
+// the image's last group and wrote ctrl->sums.
 template <typename T, typename P, bool FLAGS, bool MARGIN, bool SPLIT, int OPT>
 __device__ __forceinline__ bool track_tile(const TrackParams& p, const int term, const int bx,
                                            const int by, const int bid) {
@@ -664,8 +664,9 @@ k_track(TrackParams p, const __grid_constant__ PairEnd end) {
 
 // Tiles of every tracking slot at one level: block -> (slot, tile, term)
 // through the block prefix, tile -> (column, row band) in the slot's image.
-// Three blocks per SM (80 registers) measured faster than four (64 registers,
-// more spill reloads) and than two columns per thread.
+// BLOCKS per SM: three (80 registers) measured faster than four (64 registers, more
+// spill reloads) and than two columns per thread, but for the launches that
+// launch_track_batch names.
 // FLAGS (parity entry only): the same kernel that also or-s each pixel's
 // validity bits into a.flags (the slot's level image, zeroed before the launch).
 template <typename T, typename P, int OPT, bool FLAGS, bool MARGIN, int BLOCKS>
@@ -770,9 +771,12 @@ cudaError_t launch_track_batch(const BatchArgs& a, int blocks, int rows, bool fp
   // A launch that nothing else shares the GPU with and that is a little larger than one
   // wave at three blocks per SM runs at four (64 registers, some spills) when its tiles
   // are short: the second wave would hold back the step behind it, which starts once
-  // every block has started (600 blocks of one row: 320x240 490 -> 465 us per frame,
-  // 640x480 591 -> 577).  With long tiles the spills cost more than the wave (480 blocks
-  // of 16 rows: 1277x717 725 -> 801, 12 x 320x240 836 -> 910).
+  // every block has started.  One camera, two levels, us per frame at three and four:
+  // 320x240 (600 blocks of one row) 486 and 463, 288x216 (486 blocks) 485 and 461, the
+  // same within 1% with FP16 maps, FP32 partials and the optional terms, alone or
+  // together (485-500 and 462-472); RGB-D only 284 and 275, 273 and 274 at 288x216.
+  // With long tiles the spills cost more than the wave (480 blocks of 16 rows: 1277x717
+  // 725 -> 801, 12 x 320x240 836 -> 910).
   const bool four = early && rows <= 2 && blocks > 3 * kNumSms && blocks <= 4 * kNumSms;
 #define DRI_TRACK_BATCH_F(T, P, F, M, B)                                                 \
   do {                                                                                   \
