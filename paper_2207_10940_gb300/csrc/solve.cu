@@ -1685,7 +1685,10 @@ __device__ bool imu_weight_and_prediction(const SolveParams& sp, Ctrl* c, BeginS
     if (t == 0) B.fail = !good;
   }
   __syncthreads();
-  const bool pd = !B.fail;
+  // One piece's six noise components cannot give the nine (r, a, v) rows a covariance of
+  // full rank: its last pivots are rounding, of either sign.  (Gyro only: the rotation
+  // rows alone.)
+  const bool pd = !B.fail && (gyro || B.W.np > 1);
   if (warp > 0) {
     for (int idx = tid - 32; idx < 18 * 18; idx += kSolveThreads - 32) {
       const int r = idx / 18, q = idx % 18;
